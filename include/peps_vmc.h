@@ -390,7 +390,9 @@ typedef struct {
   int stage_kb;    /* shared memory of the pipelined kernel's stage ring per CTA, KB (32..200;
                       0 in peps_set_tune keeps the current value) */
   int trunc_threads; /* threads of a Jacobi truncation block whose matrix fits in shared
-                        memory: 32, 64, 128 or 256 (0 in peps_set_tune keeps the value) */
+                        memory: 32, 128 or 256, or 64 (the default) for the kernel's own choice
+                        by the size and number of the matrices (0 in peps_set_tune keeps the
+                        value) */
 } peps_tune;
 int peps_autotune(peps_ctx* ctx, int reps, peps_tune* out);
 /* Sets the batched engine's launch shapes (every field of `t` but the times) for this

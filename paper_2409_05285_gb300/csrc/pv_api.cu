@@ -699,10 +699,11 @@ int init_runner_t(peps_ctx* c, int sms, BatchImpl<T>* b, int Dn, const T* theta,
   const long long cD = (long long)P->chi * Dn;
   const long long cap = 2 * cD * (cD + 1);
   const size_t trunc_bytes = (size_t)cap * sizeof(T) + (size_t)(cD + 4) * (sizeof(T) + 4) + 16;
-  const bool trunc_global = trunc_bytes > 200 * 1024;   // Jacobi matrices in global memory
-  if (!trunc_global && trunc_bytes > 48 * 1024) {
-    // one cap for every context of the process, so that none lowers it under another
-    cudaError_t e = cudaFuncSetAttribute(kb_trunc<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+  const bool trunc_global = trunc_bytes > 200 * 1024;   // room for Jacobi matrices in global memory
+  {
+    cudaError_t e = jac_setup<T, T>();
+    if constexpr (std::is_same<T, float>::value)
+      if (e == cudaSuccess) e = jac_setup<double, float>();
     if (e != cudaSuccess) return fail(c, PEPS_ECUDA, std::string("cudaFuncSetAttribute: ") + cudaGetErrorString(e));
   }
   std::vector<long long> sz;
@@ -790,8 +791,6 @@ int init_runner_t(peps_ctx* c, int sms, BatchImpl<T>* b, int Dn, const T* theta,
       e = cudaFuncSetAttribute(kb_gemm_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(kb_chol<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(kb_trunc64<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     if (e != cudaSuccess) return fail(c, PEPS_ECUDA, std::string("tensor-core setup: ") + cudaGetErrorString(e));
     b->be.tc = true;
     b->be.tc_split = P->precision == PEPS_FP32;

@@ -1111,6 +1111,7 @@ inline void bond_lists(int L1, int L2, double J1, double J2, std::vector<int>& b
 
 #if defined(__CUDACC__)
 #include "pv_prof.cuh"
+#include "pv_jacobi.cuh"
 namespace pv {
 
 constexpr int BT = 256;   // threads of the per-sample blocks
@@ -1438,15 +1439,15 @@ __global__ void __launch_bounds__(NT) kb_chol(OpChol<T> op, int n) {
   }
 }
 
+// Truncation of matrices too large for shared memory (the others run in kb_jac): the Jacobi
+// matrices live in this block's slice of a global work area (cached in L2).
 template <typename T>
 __global__ void __launch_bounds__(BT) kb_trunc(OpTrunc<T> op, int n, long long cap, T* gwork) {
   __shared__ T red[32];
   __shared__ int flag;
   extern __shared__ __align__(16) unsigned char dyn[];
-  // Jacobi matrices in shared memory, or, when they do not fit (gwork given), in this
-  // block's slice of a global work area (cached in L2)
-  T* smem = gwork ? gwork + (long long)blockIdx.x * cap : (T*)dyn;
-  T* sig = gwork ? (T*)dyn : smem + cap;
+  T* smem = gwork + (long long)blockIdx.x * cap;
+  T* sig = (T*)dyn;
   int* order = (int*)(sig + op.nc + 4);
   for (int s = blockIdx.x; s < n; s += gridDim.x) {
     op(s, red, &flag, smem, cap, order, sig, BT);   // the pairing of a 256-thread block
@@ -1454,17 +1455,16 @@ __global__ void __launch_bounds__(BT) kb_trunc(OpTrunc<T> op, int n, long long c
   }
 }
 
-// The truncation of float data with a float64 working copy (rotations, singular values and
-// vectors in float64): the matrices in shared memory, or, with gwork, in this block's slice
-// of a global float64 work area.
+// The same for float data with a float64 working copy (rotations, singular values and vectors
+// in float64).
 template <typename T>
 __global__ void __launch_bounds__(BT) kb_trunc64(OpTrunc<T> op, int n, long long cap, double* gwork,
                                                  double tol) {
   __shared__ double red[32];
   __shared__ int flag;
   extern __shared__ __align__(16) unsigned char dyn[];
-  double* smem = gwork ? gwork + (long long)blockIdx.x * cap : (double*)dyn;
-  double* sig = gwork ? (double*)dyn : smem + cap;
+  double* smem = gwork + (long long)blockIdx.x * cap;
+  double* sig = (double*)dyn;
   int* order = (int*)(sig + op.nc + 4);
   for (int s = blockIdx.x; s < n; s += gridDim.x) {
     op.template run<double>(s, red, &flag, smem, order, sig, BT, tol);
@@ -1472,9 +1472,8 @@ __global__ void __launch_bounds__(BT) kb_trunc64(OpTrunc<T> op, int n, long long
   }
 }
 
-// Truncation of a tall bond (no rotations to accumulate) with its Jacobi matrix in shared
-// memory, one 1024-thread block per SM: the column pairs of a round are spread over all
-// threads and every round runs at shared-memory latency.
+// Truncation of a tall bond (no rotations to accumulate) whose matrix fits the shared memory of
+// an SM only unpadded (kb_jac pads its columns to whole vectors): one 1024-thread block per SM.
 template <typename T>
 __global__ void __launch_bounds__(1024) kb_trunc_wide(OpTrunc<T> op, int n) {
   __shared__ T red[32];
@@ -1574,8 +1573,9 @@ struct BatchTune {
   int pipelined = 1;           // tensor-core GEMM on the cp.async pipeline (kb_gemm_tc2): 0 none,
                                // 1 short vector contractions (K <= 64), 2 every vector one
   int stage_budget = 96 * 1024;   // ... bytes of copy stages per CTA
-  int trunc_threads = 64;      // threads of a Jacobi truncation block (32..256) when its
-                               // matrix is in shared memory (the same bits for each)
+  int trunc_threads = 64;      // threads of a Jacobi truncation block (32, 128, 256) when its
+                               // matrix is in shared memory (the same bits for each); 64: by
+                               // the size and number of the matrices (jac_launch)
 };
 
 // Whether two operands address the same values for every chain.
@@ -1809,55 +1809,38 @@ struct CudaBE {
     PV_KLAUNCH(prof, st, "kb_lq", lq_bytes, fl * n,
                kb_lq<T><<<gblocks(n), BT, use ? bytes : 0, st>>>(op, n, use));
   }
+  // Truncation: the matrix in the shared memory of one block (kb_jac) wherever it fits, with
+  // the lane groups jacobi() forms in a 256-thread block, or in the 1024-thread block that tall
+  // bonds take when the largest matrix of the geometry exceeds the 200 KB work area (trunc_g);
+  // larger ones on the general kernels, whose work area is global.
   void trunc(OpTrunc<T> op, int n) {
+    const int threads = tune.trunc_threads == 64 ? 0 : tune.trunc_threads;
+    const double bytes_alg = (double)n * 2.0 * op.nc * op.len * sizeof(T);
     if (trunc64) {
-      const long long need = (long long)op.nc * (op.len | 1) + (op.tall ? 0 : (long long)op.m * (op.m | 1));
-      const size_t bytes = (size_t)need * 8 + (size_t)(op.nc + 4) * (8 + sizeof(int)) + 16;
-      if (bytes <= 200 * 1024 || !trunc_g64) {
-        const int tt = tune.trunc_threads;
-        int per_sm = (int)((size_t)(227 * 1024) / (bytes + 1024));
-        per_sm = per_sm < 2048 / tt ? per_sm : 2048 / tt;
-        per_sm = per_sm < 32 ? per_sm : 32;
-        per_sm = per_sm < 1 ? 1 : per_sm;
-        const int grid = n < sms * per_sm ? n : sms * per_sm;
-        PV_KLAUNCH(prof, st, "kb_trunc", (double)n * 2.0 * op.nc * op.len * sizeof(T), 0.0,
-                   kb_trunc64<T><<<grid, tt, bytes, st>>>(op, n, need, nullptr, jtol64));
+      const JacShape s = jac_shape<double>(op.nc, op.len, op.m, op.tall, BT);
+      if (s.bytes <= (size_t)JAC_SMEM_MAX) {
+        PV_KLAUNCH(prof, st, "kb_trunc", bytes_alg, 0.0, (jac_launch<double, T>(op, n, s, jtol64, sms, threads, st)));
       } else {
         const size_t b = (size_t)(op.nc + 4) * (8 + sizeof(int)) + 16;
-        PV_KLAUNCH(prof, st, "kb_trunc", (double)n * 2.0 * op.nc * op.len * sizeof(T), 0.0,
+        PV_KLAUNCH(prof, st, "kb_trunc", bytes_alg, 0.0,
                    kb_trunc64<T><<<gblocks(n), BT, b, st>>>(op, n, trunc_cap, trunc_g64, jtol64));
       }
       return;
     }
-    if (op.tall && trunc_g) {
-      // matrices too large for the shared-memory work area of the 256-thread kernel (which
-      // would keep them in global memory): one 1024-thread block per SM holds one in shared
-      // memory; smaller ones keep eight 256-thread blocks per SM
-      const size_t wb = (size_t)op.nc * (op.len | 1) * sizeof(T) + (size_t)(op.nc + 4) * (sizeof(T) + sizeof(int)) + 16;
-      if (wb <= (size_t)trunc_wide_max) {
-        const int grid = n < sms ? n : sms;
-        PV_KLAUNCH(prof, st, "kb_trunc", (double)n * 2.0 * op.nc * op.len * sizeof(T), 0.0,
-                   kb_trunc_wide<T><<<grid, 1024, wb, st>>>(op, n));
-        return;
-      }
+    const size_t wb = (size_t)op.nc * (op.len | 1) * sizeof(T) + (size_t)(op.nc + 4) * (sizeof(T) + sizeof(int)) + 16;
+    const bool wide = op.tall && trunc_g && wb <= (size_t)trunc_wide_max;
+    const JacShape s = jac_shape<T>(op.nc, op.len, op.m, op.tall, wide ? 1024 : BT);
+    if (s.bytes <= (size_t)JAC_SMEM_MAX) {
+      PV_KLAUNCH(prof, st, "kb_trunc", bytes_alg, 0.0, (jac_launch<T, T>(op, n, s, op.jtol, sms, threads, st)));
+      return;
     }
-    if (!trunc_g) {
-      // the matrix (and, for a wide bond, its accumulated right vectors) in shared memory:
-      // as many blocks per SM as that memory and the block size allow
-      const long long need = (long long)op.nc * (op.len | 1) + (op.tall ? 0 : (long long)op.m * (op.m | 1));
-      const size_t bytes = (size_t)need * sizeof(T) + (size_t)(op.nc + 4) * (sizeof(T) + sizeof(int)) + 16;
-      const int tt = tune.trunc_threads;
-      int per_sm = (int)((size_t)(227 * 1024) / (bytes + 1024));
-      per_sm = per_sm < 2048 / tt ? per_sm : 2048 / tt;
-      per_sm = per_sm < 32 ? per_sm : 32;
-      per_sm = per_sm < 1 ? 1 : per_sm;
-      const int grid = n < sms * per_sm ? n : sms * per_sm;
-      PV_KLAUNCH(prof, st, "kb_trunc", (double)n * 2.0 * op.nc * op.len * sizeof(T), 0.0,
-                 kb_trunc<T><<<grid, tt, bytes, st>>>(op, n, need, nullptr));
+    if (wide) {
+      const int grid = n < sms ? n : sms;
+      PV_KLAUNCH(prof, st, "kb_trunc", bytes_alg, 0.0, kb_trunc_wide<T><<<grid, 1024, wb, st>>>(op, n));
       return;
     }
     size_t bytes = (size_t)(op.nc + 4) * sizeof(T) + (size_t)(op.nc + 4) * sizeof(int) + 16;
-    PV_KLAUNCH(prof, st, "kb_trunc", (double)n * 2.0 * op.nc * op.len * sizeof(T), 0.0,
+    PV_KLAUNCH(prof, st, "kb_trunc", bytes_alg, 0.0,
                kb_trunc<T><<<gblocks(n), BT, bytes, st>>>(op, n, trunc_cap, trunc_g));
   }
   // Whether an m x m Gram factorisation fits the shared memory of one kb_chol block (the
