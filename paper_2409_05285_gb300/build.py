@@ -9,7 +9,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 OUT_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT_DIR, "libpeps_vmc.so")
-SOURCES = ["pv_api.cu", "pv_serve.cu", "pv_cv.cu"]
+SOURCES = ["pv_api.cu", "pv_prog.cu", "pv_serve.cu", "pv_cv.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-I", os.path.join(ROOT, "include")]
 

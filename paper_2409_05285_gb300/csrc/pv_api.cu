@@ -330,8 +330,141 @@ struct BatchImpl : BatchIface {
   };
   bool graphs = false;
   std::map<std::tuple<int, int, long long, const void*, const void*>, Graph> gcache;
+  // Chain programs (pv_prog.cuh) by (sequence, options, chains per SM), and the site tensors
+  // they were recorded with
+  enum { SEQ_EVAL, SEQ_MC, SEQ_DOWN, SEQ_DRAW, SEQ_AMP, SEQ_OROWS };
+  std::map<std::tuple<int, int, int, const void*>, PgProgram> progs;
   BatchImpl() : run(be) {}
-  ~BatchImpl() override { drop_graphs(); }
+  ~BatchImpl() override {
+    drop_graphs();
+    drop_programs();
+  }
+  void drop_programs() {
+    for (auto& kv : progs) {
+      if (kv.second.d_ops) cudaFree(kv.second.d_ops);
+      if (kv.second.d_tab) cudaFree(kv.second.d_tab);
+    }
+    progs.clear();
+  }
+  // The program of a sequence for n chains: recorded and uploaded on first use by fn, which
+  // issues the runner's operations for one chain on the arrays of `ext`.  Null where an
+  // operation has no program form (too large for a block's shared memory): batched launches
+  // then.
+  template <typename F>
+  const PgProgram* program(int seq, int opt, int n, const std::vector<typename PgBuild<T>::Ext>& ext, F&& fn) {
+    if (N > 256 || (be.prof && be.prof->on)) return nullptr;   // profiling times every launch
+    const int q = std::min((n + be.sms - 1) / be.sms, 16);   // block shapes depend on the chains per SM
+    const auto key = std::make_tuple(seq, opt, q < 16 ? q : n, (const void*)run.theta);
+    auto it = progs.find(key);
+    if (it != progs.end()) return it->second.bad ? nullptr : &it->second;
+    PgProgram pr;
+    const double f0 = run.flops;
+    // a first recording finds the largest operation; blocks whose shared memory it exceeds get a
+    // larger share
+    int threads = 512, per_sm = 1;
+    bool sized = false;
+    for (;;) {
+      PgBuild<T> bd;
+      bd.per_sm = per_sm;
+      bd.threads = threads;
+      bd.budget = PG_SMEM / per_sm - PG_STATIC;
+      bd.ext = ext;
+      const void* sc[4] = {run.b.val, run.b.num, run.b.den, run.b.val2};
+      const void* i8[4] = {run.b.si, run.b.sj, run.b.valid, run.b.accepted};
+      for (int k = 0; k < 4; ++k) {
+        bd.sc[k] = sc[k];
+        bd.i8[k] = i8[k];
+      }
+      run.flops = 0;
+      be.rec = &bd;
+      fn();
+      be.rec = nullptr;
+      pr.flops = run.flops;
+      run.flops = f0;
+      pr.nops = (int)bd.ops.size();
+      if (!sized && !bd.bad) {
+        if (!pg_wins(n, pr.nops, pr.flops, sizeof(T) == 8)) {
+          pr.bad = true;
+          break;
+        }
+        sized = true;
+        threads = pg_threads(n, be.sms, bd.largest, bd.tc_used);
+        per_sm = std::min(512 / threads, q);
+        if (threads < 512) continue;
+      }
+      if (bd.bad && per_sm > 1) {
+        per_sm = per_sm > 4 ? per_sm / 2 : per_sm - 1;
+        continue;
+      }
+      pr.bad = bd.bad;
+      if (pr.bad) break;
+      PgOp end;
+      memset(&end, 0, sizeof(end));
+      end.kind = -1;
+      while (bd.ops.size() % PG_BLOCK) bd.ops.push_back(end);
+      pr.threads = bd.threads;
+      pr.per_sm = per_sm;
+      pr.tmem_cols = sizeof(T) == 4 ? std::max(bd.tmem, 32) : 0;
+      pr.arena = (bd.need + 127) & ~(size_t)127;
+      pr.bytes = bd.bytes;
+      const size_t ob = bd.ops.size() * sizeof(PgOp), tb = (bd.tab.size() + 4) * sizeof(int);
+      cudaError_t e = cudaMalloc((void**)&pr.d_ops, ob);
+      if (e == cudaSuccess) e = cudaMalloc((void**)&pr.d_tab, tb);
+      if (e == cudaSuccess) e = cudaMemcpy(pr.d_ops, bd.ops.data(), ob, cudaMemcpyHostToDevice);
+      if (e == cudaSuccess && !bd.tab.empty())
+        e = cudaMemcpy(pr.d_tab, bd.tab.data(), bd.tab.size() * sizeof(int), cudaMemcpyHostToDevice);
+      if (e != cudaSuccess) {   // no room: the batched launches need none
+        cudaGetLastError();
+        if (pr.d_ops) cudaFree(pr.d_ops);
+        if (pr.d_tab) cudaFree(pr.d_tab);
+        pr = PgProgram();
+        pr.bad = true;
+      }
+      break;
+    }
+    it = progs.emplace(key, pr).first;
+    return pr.bad ? nullptr : &it->second;
+  }
+  PgArgs args(int n) const {
+    PgArgs a;
+    memset(&a, 0, sizeof(a));
+    a.gbase = (char*)run.b.envD;
+    a.gint = (pgptr)run.b.envD;
+    a.n = n;
+    a.N = N;
+    a.sweep_dev = d_sweep;
+    a.jflops = run.jflops;
+    return a;
+  }
+  void exec(const PgProgram* p, const PgArgs& a) {
+    run.flops += p->flops * a.n;
+    PV_KLAUNCH(be.prof, be.st, "kb_prog", p->bytes * a.n, p->flops * a.n,
+               (pg_launch<T>(*p, a, run.jtol, be.jtol64, run.max_sweeps, run.sweeps, be.tc_err, be.sms, be.st)));
+  }
+  static typename PgBuild<T>::Ext slot(const void* p, int k) { return {(const char*)p, 1, k}; }
+
+  // log|rho| and signs (plain_amplitude) and O rows (plain_log_derivative) of n configurations
+  void amplitude(const uint8_t* S, int n, double* la, int8_t* sg) {
+    count_jacobi();
+    const PgProgram* p = program(SEQ_AMP, 0, n, {slot(S, PS_S), slot(la, PS_LA), slot(sg, PS_SG)},
+                                 [&]() { plain_amplitude(run, S, 1, la, sg); });
+    if (!p) return plain_amplitude(run, S, n, la, sg);
+    PgArgs a = args(n);
+    a.slot[PS_S] = (void*)S;
+    a.slot[PS_LA] = la;
+    a.slot[PS_SG] = sg;
+    exec(p, a);
+  }
+  void orows(const uint8_t* S, int n, T* O, long long No) {
+    count_jacobi();
+    const PgProgram* p = program(SEQ_OROWS, 0, n, {slot(S, PS_S), slot(O, PS_O)},
+                                 [&]() { plain_log_derivative(run, S, 1, O, No); });
+    if (!p) return plain_log_derivative(run, S, n, O, No);
+    PgArgs a = args(n);
+    a.slot[PS_S] = (void*)S;
+    a.slot[PS_O] = O;
+    exec(p, a);
+  }
   int* err_flag() override { return be.tc_err; }
   BatchTune& tuning() override { return be.tune; }
   bool uses_tensor_cores() const override { return be.tc; }
@@ -346,6 +479,7 @@ struct BatchImpl : BatchIface {
       be.trunc64 = on;
       if (g64) be.trunc_g64 = g64;
       drop_graphs();
+      drop_programs();
       return true;
     }
     (void)on;
@@ -412,11 +546,28 @@ struct BatchImpl : BatchIface {
     for (int off = 0; off < nb; off += chunk) {
       int n = std::min(chunk, nb - off);
       const bool cu = cached && nb <= chunk;
+      const uint8_t* S0 = S + (long long)off * N;
+      double *la0 = la ? la + off : nullptr, *es0 = es ? es + off : es_tmp, *ea0 = ea ? ea + off : ea_tmp;
+      int8_t* sg0 = sg ? sg + off : nullptr;
+      T* O0 = O ? (T*)O + (long long)off * No : nullptr;
+      std::vector<typename PgBuild<T>::Ext> ext = {slot(S0, PS_S), slot(es0, PS_ES), slot(ea0, PS_EA)};
+      if (la0) ext.push_back(slot(la0, PS_LA));
+      if (sg0) ext.push_back(slot(sg0, PS_SG));
+      if (O0) ext.push_back(slot(O0, PS_O));
+      const PgProgram* p = program(SEQ_EVAL, (cu ? 1 : 0) + (O ? 2 : 0), n, ext, [&]() {
+        run.eval(S0, 1, la0, sg0, es0, ea0, O0, No, cu);
+      });
+      PgArgs a = args(n);
+      a.slot[PS_S] = (void*)S0;
+      a.slot[PS_LA] = la0;
+      a.slot[PS_SG] = sg0;
+      a.slot[PS_ES] = es0;
+      a.slot[PS_EA] = ea0;
+      a.slot[PS_O] = O0;
       launch(std::make_tuple(0, cu ? 1 : 0, (long long)off, (const void*)S, (const void*)O),
              [&]() {
-               run.eval(S + (long long)off * N, n, la ? la + off : nullptr, sg ? sg + off : nullptr,
-                        es ? es + off : es_tmp, ea ? ea + off : ea_tmp,
-                        O ? (T*)O + (long long)off * No : nullptr, No, cu);
+               if (p) exec(p, a);
+               else run.eval(S0, n, la0, sg0, es0, ea0, O0, No, cu);
              });
     }
     flops = run.flops;
@@ -428,12 +579,22 @@ struct BatchImpl : BatchIface {
     run.sweep_dev = d_sweep;
     for (int off = 0; off < n_all; off += chunk) {
       int n = std::min(chunk, n_all - off);
+      uint8_t* S0 = S + (long long)off * N;
+      const PgProgram* pr = program(SEQ_MC, 0, n, {slot(S0, PS_S), slot(acc + off, PS_ACC), slot(prop + off, PS_PROP)},
+                                    [&]() { run.mc(S0, 1, p, seed, off, 0u, acc + off, prop + off); });
+      PgArgs a = args(n);
+      a.slot[PS_S] = S0;
+      a.slot[PS_ACC] = acc + off;
+      a.slot[PS_PROP] = prop + off;
+      a.chain0 = off;
+      a.p = p;
+      a.seed = seed;
       for (int k = 0; k < n_sweeps; ++k) {
         k_set_sweep<<<1, 1, 0, be.st>>>(d_sweep, (uint32_t)(sweep0 + k));
         if (be.prof) be.prof->launches += 1;
         launch(std::make_tuple(1, p, (long long)off, (const void*)S, (const void*)acc), [&]() {
-          run.mc(S + (long long)off * N, n, p, seed, off, (uint32_t)(sweep0 + k), acc + off,
-                 prop + off);
+          if (pr) exec(pr, a);
+          else run.mc(S0, n, p, seed, off, (uint32_t)(sweep0 + k), acc + off, prop + off);
         });
       }
     }
@@ -445,7 +606,28 @@ struct BatchImpl : BatchIface {
     count_jacobi();
     for (int off = 0; off < n_all; off += chunk) {
       const int n = std::min(chunk, n_all - off);
-      direct_draw(run, S + (long long)off * N, n, u + (long long)off * N, b_d, expo, logq + off);
+      uint8_t* S0 = S + (long long)off * N;
+      const double* u0 = u + (long long)off * N;
+      double* q0 = logq + off;
+      const std::vector<typename PgBuild<T>::Ext> ext = {slot(S0, PS_S), slot(u0, PS_U), slot(q0, PS_LOGQ)};
+      const PgProgram* pd = program(SEQ_DOWN, 0, 1, ext, [&]() { run.build_down(S0, 1); });
+      const PgProgram* pr = program(SEQ_DRAW, 0, n, ext, [&]() { direct_rows(run, S0, 1, u0, b_d, expo, q0); });
+      if (!pd || !pr) {
+        direct_draw(run, S0, n, u0, b_d, expo, q0);
+        continue;
+      }
+      PgArgs a = args(1);
+      a.slot[PS_S] = S0;
+      a.slot[PS_U] = (void*)u0;
+      a.slot[PS_LOGQ] = q0;
+      a.b_d = b_d;
+      a.expo = expo;
+      be.fill_u8(S0, 4, (long long)n * N);
+      be.setd(q0, 1, 0, 0.0, n);
+      exec(pd, a);
+      run.broadcast_down(n);
+      a.n = n;
+      exec(pr, a);
     }
     flops = run.flops;
   }
@@ -704,6 +886,7 @@ int init_runner_t(peps_ctx* c, int sms, BatchImpl<T>* b, int Dn, const T* theta,
     cudaError_t e = jac_setup<T, T>();
     if constexpr (std::is_same<T, float>::value)
       if (e == cudaSuccess) e = jac_setup<double, float>();
+    if (e == cudaSuccess) e = pg_setup<T>();
     if (e != cudaSuccess) return fail(c, PEPS_ECUDA, std::string("cudaFuncSetAttribute: ") + cudaGetErrorString(e));
   }
   std::vector<long long> sz;
@@ -1117,6 +1300,7 @@ size_t peps_footprint(const peps_params* P) {
   }
   else b += (size_t)n * ((long long)P->L1 * P->L2 * sd.ENV * real + (long long)P->L1 * (P->L2 + 1) * 4);
   b += n * 8 * 3 + 6 * Np * 8 + (real == 4 ? Np * 4 : 0) + 2 * (size_t)nch * Np * 8;   // SR
+  if (batched) b += (size_t)N * 100 * 1024;   // chain programs: about 100 records a site and sequence
   return b + (1 << 20);
 }
 
@@ -2032,9 +2216,9 @@ int famp_amplitudes(peps_famp* f, const uint8_t* dS, long long count, double* la
     for (int o2 = 0; o2 < nb; o2 += chunk) {
       const int n = std::min(chunk, nb - o2);
       if (f->b64)
-        plain_amplitude(f->b64->run, f->d_S32 + (long long)o2 * N, n, la + off + o2, sg + off + o2);
+        f->b64->amplitude(f->d_S32 + (long long)o2 * N, n, la + off + o2, sg + off + o2);
       else
-        plain_amplitude(f->b32->run, f->d_S32 + (long long)o2 * N, n, la + off + o2, sg + off + o2);
+        f->b32->amplitude(f->d_S32 + (long long)o2 * N, n, la + off + o2, sg + off + o2);
     }
     PV_KLAUNCH(&c->kprof, st, "k_fapply", 0.0, 0.0,
                k_fapply<<<(nb + 127) / 128, 128, 0, st>>>(nb, f->d_csign, sg + off, la + off));
@@ -2213,9 +2397,9 @@ int famp_orows(peps_famp* f, int nb) {
   for (int off = 0; off < nb; off += chunk) {
     const int n = std::min(chunk, nb - off);
     if (f->b64)
-      plain_log_derivative(f->b64->run, f->d_S32 + (long long)off * N, n, (double*)f->d_O + (long long)off * No, No);
+      f->b64->orows(f->d_S32 + (long long)off * N, n, (double*)f->d_O + (long long)off * No, No);
     else
-      plain_log_derivative(f->b32->run, f->d_S32 + (long long)off * N, n, (float*)f->d_O + (long long)off * No, No);
+      f->b32->orows(f->d_S32 + (long long)off * N, n, (float*)f->d_O + (long long)off * No, No);
   }
   long long big = 0;
   for (int i = 0; i < N; ++i) big = std::max(big, c->ooff[i + 1] - c->ooff[i]);

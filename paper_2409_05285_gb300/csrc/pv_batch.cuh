@@ -1112,6 +1112,7 @@ inline void bond_lists(int L1, int L2, double J1, double J2, std::vector<int>& b
 #if defined(__CUDACC__)
 #include "pv_prof.cuh"
 #include "pv_jacobi.cuh"
+#include "pv_prog.cuh"
 namespace pv {
 
 constexpr int BT = 256;   // threads of the per-sample blocks
@@ -1280,16 +1281,17 @@ __global__ void __launch_bounds__(BT) kb_lq(OpLq<T> op, int n, int use_smem) {
 // a -= (2 v.a / |v|^2) v) and L[jj][j] = a_j.  The group holding row j+1 also forms that
 // row's tail norm and its reflector for step j+1, so each step costs one barrier.
 // Needs nn and ld multiples of 4.
-template <typename T, int NT>
-__global__ void __launch_bounds__(NT) kb_lq2(OpLq<T> op, int n, int ld, int G) {
+// The bits do not depend on the number of threads (a multiple of 32): a row's sums run over its
+// group of G lanes.
+template <typename T>
+__device__ __forceinline__ void lq2_matrix(const OpLq<T>& op, int s, T* Wm, T* s_alpha, T* s_vn2, int ld,
+                                           int G) {
   typedef typename std::conditional<sizeof(T) == 8, double2, float4>::type V2;
-  extern __shared__ __align__(16) unsigned char dyn[];
-  T* Wm = (T*)dyn;
-  __shared__ T s_alpha[2], s_vn2[2];
+  const int NT = blockDim.x;
   const int m = op.m, nn = op.nn, K = m < nn ? m : nn;
   const int tid = threadIdx.x, grp = tid / G, gl = tid - grp * G, ngrp = NT / G;
   const int nq = nn >> 2;   // 4-wide vectors per row
-  for (int s = blockIdx.x; s < n; s += gridDim.x) {
+  {
     const T* W = op.W + (long long)s * op.ws;
     T* Lo = op.Lf + (long long)s * op.ls;
     for (int i = tid; i < m * nn; i += NT) {
@@ -1384,58 +1386,129 @@ __global__ void __launch_bounds__(NT) kb_lq2(OpLq<T> op, int n, int ld, int G) {
   }
 }
 
-// Semidefinite Cholesky factor of each chain's m x m Gram matrix in shared memory (row
-// stride m + 1): pivots below m eps max(diag) zero their column (rank-deficient Grams).
-template <typename T, int NT = BT>
-__global__ void __launch_bounds__(NT) kb_chol(OpChol<T> op, int n) {
+template <typename T, int NT>
+__global__ void __launch_bounds__(NT) kb_lq2(OpLq<T> op, int n, int ld, int G) {
   extern __shared__ __align__(16) unsigned char dyn[];
-  T* A = (T*)dyn;
-  __shared__ T red[32];
-  __shared__ T s_piv[2];
-  const int m = op.m, ld = m + 1;
+  __shared__ T s_alpha[2], s_vn2[2];
+  for (int s = blockIdx.x; s < n; s += gridDim.x) lq2_matrix(op, s, (T*)dyn, s_alpha, s_vn2, ld, G);
+}
+
+// Semidefinite Cholesky factor of one chain's m x m Gram matrix in shared memory (row stride
+// m + 1): pivots below m eps max(diag) zero their column (rank-deficient Grams).  Only the
+// lower triangle is updated (the factor reads nothing above the diagonal).
+template <typename T>
+__device__ __forceinline__ void chol_matrix(const OpChol<T>& op, int s, T* A, T* red, T* s_piv) {
+  const int NT = blockDim.x, m = op.m, ld = m + 1;
   const T eps = sizeof(T) == 4 ? (T)1.1920929e-7 : (T)2.220446049250313e-16;
-  for (int s = blockIdx.x; s < n; s += gridDim.x) {
-    const T* G = op.G + (long long)s * op.gs;
-    T* L = op.Lf + (long long)s * op.ls;
-    T dmax = 0;
-    for (int i = threadIdx.x; i < m * m; i += NT) {
-      const int r = i / m, c = i - r * m;
-      const T v = G[i];
+  const T* G = op.G + (long long)s * op.gs;
+  T* L = op.Lf + (long long)s * op.ls;
+  const int ty = threadIdx.x >> 5, tx = threadIdx.x & 31, nw = NT >> 5;
+  T dmax = 0;
+  for (int r = ty; r < m; r += nw)
+    for (int c = tx; c < m; c += 32) {
+      const T v = G[r * m + c];
       A[r * ld + c] = v;
       if (r == c) dmax = v > dmax ? v : dmax;
     }
-    dmax = cta_max(dmax, red);
-    const T tol = (T)m * eps * dmax;
+  dmax = cta_max(dmax, red);
+  const T tol = (T)m * eps * dmax;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    const T d = A[0];
+    s_piv[0] = d > tol ? sqrt(d) : (T)0;
+  }
+  __syncthreads();
+  for (int j = 0; j < m; ++j) {
+    const T l = s_piv[j & 1], inv = l > 0 ? (T)1 / l : (T)0;
+    for (int i = j + threadIdx.x; i < m; i += NT) A[i * ld + j] = i == j ? l : A[i * ld + j] * inv;
     __syncthreads();
-    if (threadIdx.x == 0) {
-      const T d = A[0];
-      s_piv[0] = d > tol ? sqrt(d) : (T)0;
+    // trailing update, a warp per row; thread 0 updates the next diagonal entry and forms the
+    // next pivot, so a column costs two barriers
+    for (int k = j + 1 + tx; k < m; k += 32) {
+      const T lkj = A[k * ld + j];
+      int i = j + 1 + ty;
+      if (i < k) i += (k - i + nw - 1) / nw * nw;
+#pragma unroll 4
+      for (; i < m; i += nw) A[i * ld + k] -= A[i * ld + j] * lkj;
+    }
+    if (threadIdx.x == 0 && j + 1 < m) {
+      const T d = A[(j + 1) * ld + j + 1];
+      s_piv[(j + 1) & 1] = d > tol ? sqrt(d) : (T)0;
     }
     __syncthreads();
-    for (int j = 0; j < m; ++j) {
-      const T l = s_piv[j & 1], inv = l > 0 ? (T)1 / l : (T)0;
-      for (int i = j + threadIdx.x; i < m; i += NT) A[i * ld + j] = i == j ? l : A[i * ld + j] * inv;
-      __syncthreads();
-      // trailing update on a TW x TW thread grid (TW = 16 for 256 threads, 32 for 1024);
-      // thread 0 updates the next diagonal entry and forms the next pivot, so a column costs
-      // two barriers
-      constexpr int TW = NT >= 1024 ? 32 : 16;
-      const int ty = threadIdx.x / TW, tx = threadIdx.x % TW;
-      for (int i = j + 1 + ty; i < m; i += TW) {
-        const T lij = A[i * ld + j];
-        for (int k = j + 1 + tx; k < m; k += TW) A[i * ld + k] -= lij * A[k * ld + j];
+  }
+  for (int r = ty; r < m; r += nw)
+    for (int c = tx; c < m; c += 32) L[r * m + c] = c <= r ? A[r * ld + c] : (T)0;
+  __syncthreads();
+}
+
+// The same factor (same bits: every entry takes its updates in column order) of a matrix of at
+// most 64 rows with its entries in registers: 16 column lanes x TY row groups, thread (tx, ty)
+// holds rows ty + TY r, columns tx + 16 c.  A step publishes column j in shared memory (two
+// buffers), then every thread forms the pivot and the scaled entries it needs itself, so a column
+// costs one barrier and no shared-memory traffic for the trailing matrix.  `lc` 2 x 64 entries.
+template <typename T, int TY>
+__device__ __forceinline__ void chol64(const OpChol<T>& op, int s, T* lc, T* red) {
+  constexpr int R = 64 / TY;
+  const int m = op.m, tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  const T eps = sizeof(T) == 4 ? (T)1.1920929e-7 : (T)2.220446049250313e-16;
+  const T* G = op.G + (long long)s * op.gs;
+  T* L = op.Lf + (long long)s * op.ls;
+  T a[R][4];
+  T dmax = 0;
+#pragma unroll
+  for (int r = 0; r < R; ++r)
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const int i = ty + TY * r, k = tx + 16 * c;
+      a[r][c] = (i < m && k < m) ? G[i * m + k] : (T)0;
+      if (i == k && i < m) dmax = a[r][c] > dmax ? a[r][c] : dmax;
+    }
+  dmax = cta_max(dmax, red);
+  const T tol = (T)m * eps * dmax;
+#pragma unroll
+  for (int cj = 0; cj < 4; ++cj) {
+    for (int jj = 0; jj < 16; ++jj) {
+      const int j = cj * 16 + jj;
+      if (j >= m) break;
+      T* col = lc + (j & 1) * 64;
+      if (tx == jj) {
+#pragma unroll
+        for (int r = 0; r < R; ++r) col[ty + TY * r] = a[r][cj];
       }
-      if (threadIdx.x == 0 && j + 1 < m) {
-        const T d = A[(j + 1) * ld + j + 1];
-        s_piv[(j + 1) & 1] = d > tol ? sqrt(d) : (T)0;
-      }
       __syncthreads();
+      const T d = col[j];
+      const T l = d > tol ? sqrt(d) : (T)0, inv = l > 0 ? (T)1 / l : (T)0;
+      T li[R], lk[4];
+#pragma unroll
+      for (int r = 0; r < R; ++r) li[r] = col[ty + TY * r] * inv;
+#pragma unroll
+      for (int c = 0; c < 4; ++c) lk[c] = c >= cj ? col[tx + 16 * c] * inv : (T)0;
+      if (tx == jj) {
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          const int i = ty + TY * r;
+          if (i < m) L[i * m + j] = i < j ? (T)0 : (i == j ? l : li[r]);
+        }
+      }
+#pragma unroll
+      for (int r = 0; r < R; ++r)
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+          if (c >= cj) a[r][c] -= li[r] * lk[c];
     }
-    for (int i = threadIdx.x; i < m * m; i += NT) {
-      const int r = i / m, c = i - r * m;
-      L[i] = c <= r ? A[r * ld + c] : (T)0;
-    }
-    __syncthreads();
+  }
+  __syncthreads();
+}
+
+template <typename T, int NT = BT>
+__global__ void __launch_bounds__(NT) kb_chol(OpChol<T> op, int n) {
+  extern __shared__ __align__(16) unsigned char dyn[];
+  __shared__ T red[32];
+  __shared__ T s_piv[2];
+  for (int s = blockIdx.x; s < n; s += gridDim.x) {
+    if (NT == 256 && op.m <= 64) chol64<T, 16>(op, s, (T*)dyn, red);
+    else chol_matrix(op, s, (T*)dyn, red, s_piv);
   }
 }
 
@@ -1524,19 +1597,19 @@ __global__ void kb_set(T* x, long long xs, long long off, T v, int n) {
   if (s < n) x[(long long)s * xs + off] = v;
 }
 
-__global__ void kb_fill_u8(uint8_t* x, uint8_t v, long long count) {
+static __global__ void kb_fill_u8(uint8_t* x, uint8_t v, long long count) {
   for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < count;
        k += (long long)gridDim.x * blockDim.x)
     x[k] = v;
 }
 
-__global__ void kb_bcastd(double* x, long long xs, long long len, int n) {
+static __global__ void kb_bcastd(double* x, long long xs, long long len, int n) {
   const int s = blockIdx.y + 1;
   const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (s < n && k < len) x[(long long)s * xs + k] = x[k];
 }
 
-__global__ void kb_copyd(double* x, long long xs, int dst, int src, int n) {
+static __global__ void kb_copyd(double* x, long long xs, int dst, int src, int n) {
   int s = blockIdx.x * blockDim.x + threadIdx.x;
   if (s < n) x[(long long)s * xs + dst] = x[(long long)s * xs + src];
 }
@@ -1594,10 +1667,15 @@ inline bool op_al16(const Operand<float>& o) {
   return o.site_off % 4 == 0 && o.site_sz % 4 == 0;
 }
 
-// Launch back end of the batched runner: one kernel per batched operation on `stream`.
+template <typename T>
+struct ElemDraw;
+
+// Launch back end of the batched runner: one kernel per batched operation on `stream`, or, while
+// `rec` is set, one record of the chain program being built (pv_prog.cuh).
 template <typename T, typename OT>
 struct CudaBE {
   cudaStream_t st;
+  PgBuild<T>* rec = nullptr;
   const int *bi, *bj;
   const double* bJ;
   int nb, N;
@@ -1676,6 +1754,23 @@ struct CudaBE {
   void ein(const Spec& raw, const MSpec& m, T* out, long long os, Operand<T> A, Operand<T> B,
            int n, bool exact = false) {
     GSpec gs = gemm_spec(raw);
+    if (rec) {
+      rec->bytes += ein_bytes(raw, A, B, 1);
+      if constexpr (std::is_same<T, float>::value) {
+        TcSpec t;
+        bool swap = false;
+        if (tc && tc_plan(gs, t, swap, tc_min_rows)) {
+          tc_forms(t, op_al16(swap ? B : A), op_al16(swap ? A : B), ((uintptr_t)out % 16 == 0) && os % 4 == 0);
+          t.split = (exact || tc_split) ? 1 : 0;
+          t.sym = tc_symmetric(t, op_same(A, B)) ? 1 : 0;
+          rec->tc(t, swap, out, os, A, B);
+          return;
+        }
+      }
+      if (gs.ok && gs.K <= FFMA_K_MAX) rec->fma(gs, out, os, A, B);
+      else rec->ein(m, out, os, A, B);
+      return;
+    }
     if constexpr (std::is_same<T, float>::value) {
       TcSpec t;
       bool swap = false;
@@ -1795,6 +1890,22 @@ struct CudaBE {
     const int G = op.nn >= 128 ? 16 : (op.nn >= 32 ? 8 : 4);
     const int ld = op.nn + ((G - op.nn % 32) % 32 + 32) % 32;
     const size_t bytes2 = (size_t)op.m * ld * sizeof(T);
+    if (rec) {
+      const bool two = op.nn % 4 == 0 && bytes2 <= (size_t)lq2_smem_max;
+      const size_t b1 = (size_t)op.m * op.nn * sizeof(T);
+      const bool sm = b1 <= rec->budget && b1 <= (size_t)lq_smem_max;
+      rec->fits(two ? bytes2 : (sm ? b1 : 0));
+      PgOp& o = rec->add(two ? PG_LQ2 : PG_LQ);
+      o.g.p[0] = rec->enc(op.Lf);
+      o.g.p[1] = rec->enc(op.W);
+      o.g.l[0] = op.ls;
+      o.g.l[1] = op.ws;
+      o.g.i[0] = op.m;
+      o.g.i[1] = op.nn;
+      o.g.i[2] = two ? ld : (sm ? 1 : 0);
+      o.g.i[3] = G;
+      return;
+    }
     if (op.nn % 4 == 0 && bytes2 <= (size_t)lq2_smem_max) {
       int per_sm = (int)((size_t)(227 * 1024) / (bytes2 + 1024));
       per_sm = per_sm < 2048 / LQ_THREADS ? per_sm : 2048 / LQ_THREADS;
@@ -1816,6 +1927,24 @@ struct CudaBE {
   void trunc(OpTrunc<T> op, int n) {
     const int threads = tune.trunc_threads == 64 ? 0 : tune.trunc_threads;
     const double bytes_alg = (double)n * 2.0 * op.nc * op.len * sizeof(T);
+    if (rec) {
+      const size_t wbr = (size_t)op.nc * (op.len | 1) * sizeof(T) + (size_t)(op.nc + 4) * (sizeof(T) + sizeof(int)) + 16;
+      const bool wider = op.tall && trunc_g && wbr <= (size_t)trunc_wide_max;
+      const JacShape s = trunc64 ? jac_shape<double>(op.nc, op.len, op.m, op.tall, BT)
+                                 : jac_shape<T>(op.nc, op.len, op.m, op.tall, wider ? 1024 : BT);
+      rec->fits(s.bytes + 256);
+      PgOp& o = rec->add(trunc64 ? PG_TRUNC64 : PG_TRUNC);
+      o.g.p[0] = rec->enc(op.Y);
+      o.g.p[1] = rec->enc(op.Uk);
+      o.g.p[2] = rec->enc(op.out);
+      o.g.p[3] = rec->enc(op.lsv);
+      o.g.l[0] = op.ys;
+      o.g.l[1] = op.uks;
+      o.g.l[2] = op.outs;
+      const int v[10] = {op.nc, op.len, op.m, op.tall ? 1 : 0, op.kk, op.lstride, s.G, s.lg, s.chY, s.chV};
+      for (int k = 0; k < 10; ++k) o.g.i[k] = v[k];
+      return;
+    }
     if (trunc64) {
       const JacShape s = jac_shape<double>(op.nc, op.len, op.m, op.tall, BT);
       if (s.bytes <= (size_t)JAC_SMEM_MAX) {
@@ -1850,7 +1979,17 @@ struct CudaBE {
     return bytes <= 200 * 1024 || (int)bytes <= chol_wide_max;
   }
   void chol(OpChol<T> op, int n) {
-    const size_t bytes = (size_t)op.m * (op.m + 1) * sizeof(T);
+    const size_t bytes = op.m <= 64 ? 128 * sizeof(T) : (size_t)op.m * (op.m + 1) * sizeof(T);
+    if (rec) {
+      rec->fits(rec->threads < 128 ? (size_t)op.m * (op.m + 1) * sizeof(T) : bytes);
+      PgOp& o = rec->add(PG_CHOL);
+      o.g.p[0] = rec->enc(op.G);
+      o.g.p[1] = rec->enc(op.Lf);
+      o.g.l[0] = op.gs;
+      o.g.l[1] = op.ls;
+      o.g.i[0] = op.m;
+      return;
+    }
     if (bytes > 96 * 1024 && (int)bytes <= chol_wide_max) {
       // at most one block fits per SM: 1024 threads share the trailing updates
       const int grid = n < sms ? n : sms;
@@ -1863,10 +2002,51 @@ struct CudaBE {
                (double)op.m * op.m * op.m / 3.0 * n,
                kb_chol<T><<<gblocks(n), BT, bytes, st>>>(op, n));
   }
-  void norm(OpNorm<T> op, int n) { PV_KLAUNCH(prof, st, "kb_norm", 0.0, 0.0, kb_norm<T><<<gblocks(n), BT, 0, st>>>(op, n)); }
-  void dot(OpDot<T> op, int n) { PV_KLAUNCH(prof, st, "kb_dot", 0.0, 0.0, kb_dot<T><<<gx(n, 8), 256, 0, st>>>(op, n)); }
-  void set(T* x, long long xs, long long off, T v, int n) { PV_KLAUNCH(prof, st, "kb_set", 0.0, 0.0, kb_set<T><<<gx(n, 256), 256, 0, st>>>(x, xs, off, v, n)); }
+  void norm(OpNorm<T> op, int n) {
+    if (rec) {
+      PgOp& o = rec->add(PG_NORM);
+      o.g.p[0] = rec->enc(op.x);
+      o.g.p[1] = rec->enc(op.lsv);
+      o.g.l[0] = op.xs;
+      o.g.l[1] = op.len;
+      o.g.i[0] = op.lstride;
+      return;
+    }
+    PV_KLAUNCH(prof, st, "kb_norm", 0.0, 0.0, kb_norm<T><<<gblocks(n), BT, 0, st>>>(op, n));
+  }
+  void dot(OpDot<T> op, int n) {
+    if (rec) {
+      PgOp& o = rec->add(PG_DOT);
+      o.g.p[0] = rec->enc(op.a);
+      o.g.p[1] = rec->enc(op.b);
+      o.g.p[2] = rec->enc(op.out);
+      o.g.l[0] = op.as;
+      o.g.l[1] = op.bs;
+      o.g.l[2] = op.len;
+      return;
+    }
+    PV_KLAUNCH(prof, st, "kb_dot", 0.0, 0.0, kb_dot<T><<<gx(n, 8), 256, 0, st>>>(op, n));
+  }
+  void set(T* x, long long xs, long long off, T v, int n) {
+    if (rec) {
+      PgOp& o = rec->add(PG_SET);
+      o.g.p[0] = rec->enc(x);
+      o.g.l[0] = xs;
+      o.g.l[1] = off;
+      o.g.d = (double)v;
+      return;
+    }
+    PV_KLAUNCH(prof, st, "kb_set", 0.0, 0.0, kb_set<T><<<gx(n, 256), 256, 0, st>>>(x, xs, off, v, n));
+  }
   void setd(double* x, long long xs, long long off, double v, int n) {
+    if (rec) {
+      PgOp& o = rec->add(PG_SETD);
+      o.g.p[0] = rec->enc(x);
+      o.g.l[0] = xs;
+      o.g.l[1] = off;
+      o.g.d = v;
+      return;
+    }
     PV_KLAUNCH(prof, st, "kb_set", 0.0, 0.0, kb_set<double><<<gx(n, 256), 256, 0, st>>>(x, xs, off, v, n));
   }
   // x[s][0..len) = x[0][0..len) for s = 1..n-1
@@ -1876,30 +2056,104 @@ struct CudaBE {
     PV_KLAUNCH(prof, st, "kb_copyd", 0.0, 0.0, kb_bcastd<<<g, 128, 0, st>>>(x, xs, len, n));
   }
   void copyd(double* x, long long xs, int dst, int src, int n) {
+    if (rec) {
+      PgOp& o = rec->add(PG_COPYD);
+      o.g.p[0] = rec->enc(x);
+      o.g.l[0] = xs;
+      o.g.i[0] = dst;
+      o.g.i[1] = src;
+      return;
+    }
     PV_KLAUNCH(prof, st, "kb_copyd", 0.0, 0.0, kb_copyd<<<gx(n, 256), 256, 0, st>>>(x, xs, dst, src, n));
   }
   void copy_masked(T* dst, long long ds, const T* src, long long ss, long long len,
                    const int8_t* mask, int n) {
+    if (rec) {
+      PgOp& o = rec->add(PG_COPY);
+      o.g.p[0] = rec->enc(dst);
+      o.g.p[1] = rec->enc(src);
+      o.g.l[0] = ds;
+      o.g.l[1] = ss;
+      o.g.l[2] = len;
+      o.g.i[0] = mask ? rec->sel(mask) : -1;
+      return;
+    }
     dim3 g(gx(len, 256), n);
     PV_KLAUNCH(prof, st, "kb_copy", 0.0, 0.0, kb_copy<T><<<g, 256, 0, st>>>(dst, ds, src, ss, len, mask, n));
   }
   void diag(const uint8_t* S, int n, double* es, double* ea) {
+    if (rec) {
+      PgOp& o = rec->add(PG_DIAG);
+      o.g.p[0] = rec->enc(bi);
+      o.g.p[1] = rec->enc(bj);
+      o.g.p[2] = rec->enc(bJ);
+      o.g.i[0] = nb;
+      return;
+    }
     PV_KLAUNCH(prof, st, "kb_elem_diag", 0.0, 0.0, kb_elem<<<gx(n, 128), 128, 0, st>>>(ElemDiag{S, N, nb, bi, bj, bJ, es, ea}, n));
   }
   void amp(const T* val, long long vs, const double* lsd, int lstride, double* la, int8_t* sg, int n) {
+    if (rec) {
+      PgOp& o = rec->add(PG_AMP);
+      o.g.p[0] = rec->enc(val);
+      o.g.p[1] = rec->enc(lsd);
+      o.g.l[0] = vs;
+      o.g.i[0] = lstride;
+      return;
+    }
     PV_KLAUNCH(prof, st, "kb_elem_amp", 0.0, 0.0, kb_elem<<<gx(n, 128), 128, 0, st>>>(ElemAmp<T>{val, vs, lsd, lstride, la, sg}, n));
   }
   void writeO(OT* O, long long No, long long o_off, const T* env, long long es, long long sz,
               const T* val, long long vs, int n) {
+    if (rec) {
+      PgOp& o = rec->add(PG_O);
+      o.g.p[0] = rec->enc(env);
+      o.g.p[1] = rec->enc(val);
+      o.g.l[0] = No;
+      o.g.l[1] = o_off;
+      o.g.l[2] = es;
+      o.g.l[3] = vs;
+      o.g.l[4] = sz;
+      return;
+    }
     dim3 g(gx(sz, 256), n);
     PV_KLAUNCH(prof, st, "kb_O", 0.0, 0.0, kb_O<T, OT><<<g, 256, 0, st>>>(O, No, o_off, env, es, sz, val, vs, n));
   }
-  void sel(ElemSel f, int n) { PV_KLAUNCH(prof, st, "kb_elem_sel", 0.0, 0.0, kb_elem<<<gx(n, 128), 128, 0, st>>>(f, n)); }
+  void sel(ElemSel f, int n) {
+    if (rec) {
+      PgOp& o = rec->add(PG_SEL);
+      o.g.i[0] = f.i;
+      o.g.i[1] = f.j;
+      o.g.i[2] = f.kind;
+      return;
+    }
+    PV_KLAUNCH(prof, st, "kb_elem_sel", 0.0, 0.0, kb_elem<<<gx(n, 128), 128, 0, st>>>(f, n));
+  }
   void ratio(const T* num, const T* den, long long dens, const int8_t* valid, double coef,
              double* e, int n) {
+    if (rec) {
+      PgOp& o = rec->add(PG_RATIO);
+      o.g.p[0] = rec->enc(num);
+      o.g.p[1] = rec->enc(den);
+      o.g.p[2] = rec->enc(e);
+      o.g.l[0] = dens;
+      o.g.d = coef;
+      return;
+    }
     PV_KLAUNCH(prof, st, "kb_elem_ratio", 0.0, 0.0, kb_elem<<<gx(n, 128), 128, 0, st>>>(ElemRatio<T>{num, den, dens, valid, coef, e}, n));
   }
-  void accept(ElemAccept<T> f, int n) { PV_KLAUNCH(prof, st, "kb_elem_accept", 0.0, 0.0, kb_elem<<<gx(n, 128), 128, 0, st>>>(f, n)); }
+  void accept(ElemAccept<T> f, int n) {
+    if (rec) {
+      PgOp& o = rec->add(PG_ACCEPT);
+      o.g.p[0] = rec->enc(f.num);
+      o.g.p[1] = rec->enc(f.den);
+      o.g.i[0] = f.i;
+      o.g.i[1] = f.j;
+      o.g.i[2] = (int)f.id;
+      return;
+    }
+    PV_KLAUNCH(prof, st, "kb_elem_accept", 0.0, 0.0, kb_elem<<<gx(n, 128), 128, 0, st>>>(f, n));
+  }
   // direct sampling (pv_direct.cuh): configuration fill, the candidate selector of every
   // chain, and one draw
   void fill_u8(uint8_t* x, uint8_t v, long long count) {
@@ -1907,10 +2161,21 @@ struct CudaBE {
     PV_KLAUNCH(prof, st, "kb_fill", 0.0, 0.0, kb_fill_u8<<<(unsigned)(g > 0 ? g : 1), 256, 0, st>>>(x, v, count));
   }
   void set_i8(int8_t* x, int8_t v, int n) {
+    if (rec) {
+      PgOp& o = rec->add(PG_SETI8);
+      o.g.i[0] = rec->sel(x);
+      o.g.i[1] = v;
+      return;
+    }
     PV_KLAUNCH(prof, st, "kb_set", 0.0, 0.0, kb_set<int8_t><<<gx(n, 256), 256, 0, st>>>(x, 1, 0, v, n));
   }
-  template <typename F>
-  void draw(F f, int n) { PV_KLAUNCH(prof, st, "kb_elem_draw", 0.0, 0.0, kb_elem<<<gx(n, 128), 128, 0, st>>>(f, n)); }
+  void draw(ElemDraw<T> f, int n) {
+    if (rec) {
+      rec->add(PG_DRAW).g.i[0] = f.i;
+      return;
+    }
+    PV_KLAUNCH(prof, st, "kb_elem_draw", 0.0, 0.0, kb_elem<<<gx(n, 128), 128, 0, st>>>(f, n));
+  }
 };
 
 }  // namespace pv

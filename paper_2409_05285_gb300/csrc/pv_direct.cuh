@@ -98,19 +98,13 @@ struct ElemDraw {
   }
 };
 
-// One direct draw of every chain.  `run` is a BatchRunner built for bond dimension D^2 over
-// double-layer tensors (its theta and toff); S [n][N] is overwritten with the samples (local
-// indices 0..3), logq [n] receives log q(S).
+// The rows of a draw: S all summed and the down environments built.
 template <typename T, typename BE, typename OT>
-void direct_draw(BatchRunner<T, BE, OT>& run, uint8_t* S, int n, const double* u, double b_d,
+void direct_rows(BatchRunner<T, BE, OT>& run, uint8_t* S, int n, const double* u, double b_d,
                  double expo, double* logq) {
   BE& be = run.be;
   auto& b = run.b;
   const int L1 = run.L1, L2 = run.L2, N = run.N;
-  be.fill_u8(S, 4, (long long)n * N);   // every site summed
-  be.setd(logq, 1, 0, 0.0, n);
-  run.build_down(S, 1);   // every chain's down environments are the same: build one, copy
-  run.broadcast_down(n);
   run.trivial(run.uprow(0), b.sU, n);
   be.setd(b.lsU, 1, 0, 0.0, n);
   T* cand[4] = {b.val, b.num, b.den, b.val2};
@@ -137,6 +131,21 @@ void direct_draw(BatchRunner<T, BE, OT>& run, uint8_t* S, int n, const double* u
     if (r + 1 < L1)
       run.compress(run.uprow(r), b.sU, run.shp.up[r], false, r, S, run.uprow(r + 1), b.sU, b.lsU, 1, n);
   }
+}
+
+// One direct draw of every chain.  `run` is a BatchRunner built for bond dimension D^2 over
+// double-layer tensors (its theta and toff); S [n][N] is overwritten with the samples (local
+// indices 0..3), logq [n] receives log q(S).
+template <typename T, typename BE, typename OT>
+void direct_draw(BatchRunner<T, BE, OT>& run, uint8_t* S, int n, const double* u, double b_d,
+                 double expo, double* logq) {
+  BE& be = run.be;
+  const int N = run.N;
+  be.fill_u8(S, 4, (long long)n * N);   // every site summed
+  be.setd(logq, 1, 0, 0.0, n);
+  run.build_down(S, 1);   // every chain's down environments are the same: build one, copy
+  run.broadcast_down(n);
+  direct_rows(run, S, n, u, b_d, expo, logq);
 }
 
 }  // namespace pv

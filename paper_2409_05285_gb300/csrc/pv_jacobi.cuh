@@ -145,12 +145,13 @@ __device__ __forceinline__ bool jac_pair(int rnd, int pr, int np, int nc, int& p
 // T: working type; ST: storage type of Y, U and the environment.  CH: 16-byte vectors per lane
 // and column held in registers (at least chY), or 0 to read the columns again for the rotation
 // (columns too long for registers).
-template <typename T, typename ST, int CH, int TT, int MAXT>
-__global__ void __launch_bounds__(MAXT, MAXT == 256 ? 2 : 1) kb_jac(OpTrunc<ST> op, int n, int G, int lg, int chY, int chV, T tol) {
+// The whole block works on matrix s; `dyn` is its shared work area (JacShape::bytes), `red` 32
+// shared entries.
+template <typename T, typename ST, int CH, int TT>
+__device__ __forceinline__ void jac_matrix(const OpTrunc<ST>& op, int s, unsigned char* dyn, T* red, int G,
+                                           int lg, int chY, int chV, T tol) {
   constexpr int VW = 16 / sizeof(T);
   constexpr int R = CH > 0 ? CH * VW : 1;
-  extern __shared__ __align__(16) unsigned char dyn[];
-  __shared__ T red[32];
   const int nc = op.nc, len = op.len, m = op.m, kk = op.kk;
   const bool tall = op.tall;
   const int tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31, warp = tid >> 5, nwarp = nthr >> 5;
@@ -175,7 +176,7 @@ __global__ void __launch_bounds__(MAXT, MAXT == 256 ? 2 : 1) kb_jac(OpTrunc<ST> 
                           : (TT == 2 ? ((gl & (G >> 1)) ? 1 : 0) : 0);
   const bool writer = (gl & ((TT == 4 ? G >> 2 : (TT == 2 ? G >> 1 : G)) - 1)) == 0;
 
-  for (int s = blockIdx.x; s < n; s += gridDim.x) {
+  {
     const ST* Ys = op.Y + (long long)s * op.ys;
     for (int j = warp; j < nc; j += nwarp)
       for (int i = lane; i < ldy; i += 32) Y[j * ldy + pos(i)] = i < len ? (T)Ys[(long long)j * len + i] : (T)0;
@@ -413,6 +414,14 @@ __global__ void __launch_bounds__(MAXT, MAXT == 256 ? 2 : 1) kb_jac(OpTrunc<ST> 
     }
     __syncthreads();
   }
+}
+
+template <typename T, typename ST, int CH, int TT, int MAXT>
+__global__ void __launch_bounds__(MAXT, MAXT == 256 ? 2 : 1) kb_jac(OpTrunc<ST> op, int n, int G, int lg,
+                                                                    int chY, int chV, T tol) {
+  extern __shared__ __align__(16) unsigned char dyn[];
+  __shared__ T red[32];
+  for (int s = blockIdx.x; s < n; s += gridDim.x) jac_matrix<T, ST, CH, TT>(op, s, dyn, red, G, lg, chY, chV, tol);
 }
 
 constexpr int JAC_SMEM_MAX = 220 * 1024;   // dynamic shared memory the kernels are configured for

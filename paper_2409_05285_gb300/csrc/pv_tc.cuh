@@ -208,18 +208,26 @@ __device__ __forceinline__ unsigned long long tc_now() {
   return t;
 }
 
-// Waits for the phase `parity` of an mbarrier to complete; false after TC_WAIT_NS.
+__device__ __forceinline__ bool tc_try_wait(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}\n"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  return ok;
+}
+
+// Waits for the phase `parity` of an mbarrier to complete; false after TC_WAIT_NS.  The timer is
+// read only when the first attempts have failed: reading it costs more than a tile's MMAs.
 __device__ __forceinline__ bool tc_wait(uint32_t bar, uint32_t parity) {
+  for (int i = 0; i < 1024; ++i)
+    if (tc_try_wait(bar, parity)) return true;
   const unsigned long long t0 = tc_now();
   for (;;) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}\n"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    if (ok) return true;
+    for (int i = 0; i < 64; ++i)
+      if (tc_try_wait(bar, parity)) return true;
     if (tc_now() - t0 > TC_WAIT_NS) return false;
   }
 }

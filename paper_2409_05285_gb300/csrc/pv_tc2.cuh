@@ -131,7 +131,7 @@ __device__ __forceinline__ void tc2_chunk(float* dst, float* dlo, const float* _
   }
 }
 
-__global__ void __launch_bounds__(TC_THREADS) kb_gemm_tc2(TcSpec t, float* C, long long cs,
+static __global__ void __launch_bounds__(TC_THREADS) kb_gemm_tc2(TcSpec t, float* C, long long cs,
                                                           Operand<float> P, Operand<float> Q, int n,
                                                           int tilesN, int* err) {
   extern __shared__ __align__(16) unsigned char dyn[];
