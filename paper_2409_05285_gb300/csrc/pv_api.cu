@@ -1234,7 +1234,7 @@ int peps_init(const peps_params* Pin, void* stream, peps_ctx** out) {
   if ((rc = dalloc(c, &c->d_part2, (size_t)c->nch * c->Np * sizeof(double)))) return bail(rc);
   if ((rc = dalloc(c, &c->d_bp1, c->nvb * sizeof(double)))) return bail(rc);
   if ((rc = dalloc(c, &c->d_bp2, c->nvb * sizeof(double)))) return bail(rc);
-  if ((rc = dalloc(c, &c->d_ypart, c->nyb * sizeof(double)))) return bail(rc);
+  if ((rc = dalloc(c, &c->d_ypart, 2 * c->nyb * sizeof(double)))) return bail(rc);
   if ((rc = dalloc(c, &c->d_sc, sizeof(SRScalars)))) return bail(rc);
   if (P->block_mode == PEPS_BLOCKS_BATCHED) {
     if ((rc = make_batch(c, sms))) return bail(rc);
@@ -1664,9 +1664,39 @@ int peps_sr_step(peps_ctx* c, double tau, double eps, int max_cg, double cg_tol,
   const bool fused = c->cg_mode == 1;
   (void)gv_rows;
   const int ov_blocks = c->nyb;
+  // small problems: the whole loop in one cooperative launch (same bits).  Measured per
+  // iteration, launched / one launch: 4x4 D=2, 2000 samples float64 90 / 41 us, 64 samples TF32
+  // 55 / 24 us.  From about 4e6 row entries the two passes over the rows take as long as the
+  // launches.
+  const size_t cgs_smem = (size_t)5 * Np * sizeof(double) + (size_t)3 * No * sizeof(int);
+  const bool small = c->cg_mode == 0 && max_cg > 0 && Np <= CGS_NP_MAX && (double)n * No <= 4e6 &&
+                     cgs_smem <= (size_t)180 * 1024;
+  if (small) {
+    PV_CUDA(c, cudaMemsetAsync(c->d_gvbar, 0, 2 * sizeof(unsigned), s));
+    int n_ = n, N_ = c->N, Np_ = (int)Np, nch_ = c->nch;
+    long long No_ = No;
+    const void* Op = o64 ? (const void*)c->d_O64 : (const void*)c->d_O;
+    const uint8_t* Sp = c->d_S;
+    const int* o2s = c->d_o2site;
+    const long long *tof = c->d_toff, *oof = c->d_ooff;
+    const double *wp = c->d_w, *obp = c->d_obar, *gp = c->d_g, *op0 = c->d_bp2;
+    double *xp = c->d_x, *yp = c->d_y, *ypp = c->d_ypart, *pp = c->d_part;
+    SRScalars* scp = c->d_sc;
+    unsigned* barp = c->d_gvbar;
+    int* errp = c->d_gverr;
+    void* args[] = {&n_, &N_, &No_, &Np_, &nch_, &Op, &Sp, &o2s, &tof, &oof, &wp, &obp, &gp, &op0,
+                    &xp, &yp, &ypp, &pp, &scp, &barp, &errp};
+    const bool vec = !fp64(c) && c->o_vec4;
+    const void* fn = vec ? (o64 ? (const void*)k_cg_small<double, true> : (const void*)k_cg_small<float, true>)
+                         : (fp64(c) ? (const void*)k_cg_small<double, false> : (const void*)k_cg_small<float, false>);
+    const int work = (int)std::max<long long>(ov_blocks, (No + 31) / 32 * c->nch);
+    PV_CUDA(c, cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 180 * 1024));
+    PV_KLAUNCH(&c->kprof, s, "k_cg_small", 0.0, 4.0 * (double)n * No * max_cg,
+               PV_CUDA(c, cudaLaunchCooperativeKernel(fn, dim3(std::min(work, c->gv_grid)), dim3(SR_THREADS), args, cgs_smem, s)));
+  }
   dim3 cgrid_y((unsigned)((No + SR_THREADS - 1) / SR_THREADS), (unsigned)c->nch);
   dim3 cgrid4_y((unsigned)((No / 4 + SR_THREADS - 1) / SR_THREADS), (unsigned)c->nch);
-  for (int it = 0; it < max_cg; ++it) {
+  for (int it = 0; it < max_cg && !small; ++it) {
     if (!fused) {
       // y_i = w_i (O_i.p - obar.p), then the column sums part = sum_i y_i O_i, then q
       const double ob = (double)n * No * (fp64(c) || o64 ? 8.0 : 4.0);

@@ -778,6 +778,298 @@ __global__ void __launch_bounds__(GV_THREADS) k_gv(
   if (tid == 0) pqpart[b] = pq;
 }
 
+// ---------------------------------------------------------------- CG of small problems
+//
+// The whole CG loop in one cooperative launch for problems whose vectors fit in shared memory
+// and whose passes take a few microseconds: launched one by one, the six kernels of an iteration
+// cost their launches.  Every block keeps x, r, p, q and obar and forms the vector updates
+// itself, so an iteration needs two grid barriers (after the y_i, after the column sums).  The
+// sums keep the order of the separate kernels' blocks of SR_THREADS: the same bits.
+// What bounds an iteration is float64 issue, 67 cycles of a quarter SM per warp instruction on
+// GB300, so work that one warp can do is not repeated by the others (block sums are finished
+// by one thread, scalars formed once), and a column sum is spread over a block: eight warps load
+// the chunk's 32 columns (and, for the unfused form, multiply), four warps add, one per state.
+// `VEC`: the rounding of the 16-byte forms (k_ov_f32v, k_colsum1_f32v: fused multiply-adds), else
+// of k_ov and k_colsum1 (product rounded before it is added).  The barrier waits are bounded
+// (GV_WAIT_NS): a wait that runs out raises *err and every block returns.
+// Measured per iteration at 4x4 D=2 (launched in brackets): 41 us at 2000 float64 samples (90), 24 us
+// at 64 samples (55).
+constexpr int CGS_NP_MAX = 4096;   // parameters
+constexpr int CGS_NVB = CGS_NP_MAX / SR_THREADS;
+
+// bar counts arrivals (zero at launch); k: barriers passed before.  False when a wait ran out.
+__device__ __forceinline__ bool cgs_barrier(unsigned* bar, unsigned k, int* err, int* ok_sh) {
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    int ok = 1;
+    const unsigned target = (k + 1) * gridDim.x;
+    __threadfence();
+    atomicAdd(bar, 1u);
+    unsigned v;
+    for (int i = 0;; ++i) {
+      asm volatile("ld.acquire.gpu.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
+      if (v >= target || i == 4096) break;
+    }
+    if (v < target) {
+      const unsigned long long t0 = gv_now();
+      for (;;) {
+        asm volatile("ld.acquire.gpu.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
+        if (v >= target) break;
+        if (*(volatile int*)err || gv_now() - t0 > GV_WAIT_NS) {
+          atomicOr(err, 1);
+          ok = 0;
+          break;
+        }
+      }
+    }
+    *ok_sh = ok;
+  }
+  __syncthreads();
+  return *ok_sh != 0;
+}
+
+struct CgsShared {
+  double wsum[CGS_NVB][8];       // warp sums of the vector blocks
+  double vpart[CGS_NVB];
+  double yc[OTV_CHUNK], X[OTV_CHUNK][33];
+  double s_obp, s_sumy, s_alpha, s_beta, s_rr;
+  uint8_t st[OTV_CHUNK][32];
+  int ok, done;
+};
+
+// blk_sum_parts(vpart, nvb <= 32) by the first warp.
+__device__ __forceinline__ double cgs_parts(const double* vpart, int nvb, int lane) {
+  double v = lane < nvb ? 0.0 + vpart[lane] : 0.0;
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+template <typename OT, bool VEC>
+__global__ void __launch_bounds__(SR_THREADS) k_cg_small(
+    int n, int N, long long No, int Np, int nch, const OT* __restrict__ O, const uint8_t* __restrict__ S,
+    const int* __restrict__ o2site, const long long* __restrict__ toff, const long long* __restrict__ ooff,
+    const double* __restrict__ w, const double* __restrict__ obar_g, const double* __restrict__ g,
+    const double* __restrict__ obpart0, double* __restrict__ x_g, double* __restrict__ y,
+    double* __restrict__ ypart, double* __restrict__ part, SRScalars* sc, unsigned* bar, int* err) {
+  extern __shared__ double cgs[];
+  __shared__ CgsShared sh;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int nvb = (Np + SR_THREADS - 1) / SR_THREADS, nyb = (n + 7) / 8;
+  double *x = cgs, *r = x + Np, *p = r + Np, *q = p + Np, *ob = q + Np;
+  int* base = (int*)(ob + Np);   // per column: theta index of state 0; then the site's slice length
+  int* slen = base + No;
+  int* site = slen + No;
+  const int ncw = (int)((No + 31) / 32);
+  for (int t = tid; t < Np; t += SR_THREADS) {
+    x[t] = 0.0;
+    r[t] = p[t] = g[t];
+    ob[t] = obar_g[t];
+  }
+  for (int o = tid; o < (int)No; o += SR_THREADS) {
+    const int j = o2site[o];
+    base[o] = (int)(toff[j] + (o - ooff[j]));
+    slen[o] = (int)(ooff[j + 1] - ooff[j]);
+    site[o] = j;
+  }
+  for (int i = tid; i < nvb; i += SR_THREADS) sh.vpart[i] = obpart0[i];
+  const double tol = sc->tol, gnorm = sc->gnorm, eps = sc->eps;
+  const int maxit = sc->maxit;
+  int iters = sc->iters;
+  if (tid == 0) {
+    sh.s_rr = sc->rr;
+    sh.done = sc->done;
+  }
+  unsigned nbar = 0;
+  __syncthreads();
+  while (!sh.done) {
+    // y_i = w_i (O_i . p - obar . p); the partial sums alternate between two buffers (a block may
+    // be an iteration's vector part ahead of another)
+    double* yp = ypart + (iters & 1) * nyb;
+    if (warp == 0) {
+      const double v = cgs_parts(sh.vpart, nvb, lane);
+      if (lane == 0) sh.s_obp = v;
+    }
+    __syncthreads();
+    const double obp = sh.s_obp;
+    for (int vb = blockIdx.x; vb < nyb; vb += gridDim.x) {
+      const int i = vb * 8 + warp;
+      double yi = 0;
+      if (i < n) {
+        const OT* row = O + (long long)i * No;
+        const uint8_t* Si = S + (long long)i * N;
+        double acc = 0;
+        if constexpr (VEC) {
+          const int nq = (int)(No >> 2);
+          for (int k = lane; k < nq; k += 32) {
+            const int o = k << 2;
+            const double* pp = p + base[o] + (int)Si[site[o]] * slen[o];
+            const OV4 v = ov_ld4(row + o);
+            acc += v.x * pp[0] + v.y * pp[1] + v.z * pp[2] + v.w * pp[3];
+          }
+        } else {
+          // site by site, as k_ov: a lane adds its entries of site j before those of site j + 1
+          for (int o0 = 0; o0 < (int)No;) {
+            const int sz = slen[o0], t0 = base[o0] + (int)Si[site[o0]] * sz;
+            for (int k = lane; k < sz; k += 32) acc += (double)row[o0 + k] * p[t0 + k];
+            o0 += sz;
+          }
+        }
+        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        yi = w[i] * (acc - obp);
+        if (lane == 0) y[i] = yi;
+      }
+      if (lane == 0) sh.wsum[0][warp] = yi;
+      __syncthreads();
+      if (tid == 0) {
+        double s = 0;
+        for (int k = 0; k < 8; ++k) s += sh.wsum[0][k];
+        yp[vb] = s;
+      }
+      __syncthreads();
+    }
+    if (!cgs_barrier(bar, nbar++, err, &sh.ok)) return;
+    // column sums of y_i O_i per state and chunk of samples, 32 columns at a time
+    for (int u = blockIdx.x; u < ncw * nch; u += gridDim.x) {
+      const int ch = u / ncw, o = (u - ch * ncw) * 32 + lane;
+      const int i0 = ch * OTV_CHUNK, ni = min(n - i0, OTV_CHUNK);
+      __syncthreads();
+      for (int i = tid; i < ni; i += SR_THREADS) sh.yc[i] = __ldcg(y + i0 + i);
+      const bool on = o < (int)No;
+      const int j = on ? site[o] : 0;
+      double v[OTV_CHUNK / 8];
+      uint8_t st[OTV_CHUNK / 8];
+#pragma unroll
+      for (int m = 0; m < OTV_CHUNK / 8; ++m) {
+        const int k = warp + 8 * m;
+        v[m] = 0.0;
+        st[m] = 255;
+        if (on && k < ni) {
+          v[m] = (double)O[(long long)(i0 + k) * No + o];
+          st[m] = S[(long long)(i0 + k) * N + j];
+        }
+      }
+      __syncthreads();
+#pragma unroll
+      for (int m = 0; m < OTV_CHUNK / 8; ++m) {
+        const int k = warp + 8 * m;
+        if (k < ni) {
+          sh.X[k][lane] = VEC ? v[m] : __dmul_rn(sh.yc[k], v[m]);
+          sh.st[k][lane] = st[m];
+        }
+      }
+      __syncthreads();
+      if (warp < 4) {   // one warp per state
+        double a = 0.0;
+#pragma unroll 8
+        for (int k = 0; k < ni; ++k)
+          if (sh.st[k][lane] == warp) a = VEC ? fma(sh.yc[k], sh.X[k][lane], a) : __dadd_rn(a, sh.X[k][lane]);
+        if (on) part[(long long)ch * Np + base[o] + warp * slen[o]] = a;
+      }
+    }
+    if (!cgs_barrier(bar, nbar++, err, &sh.ok)) return;
+    // q = sum_ch part - (sum y) obar + eps p, p.q
+    {
+      double ys = 0;
+      for (int i = tid; i < nyb; i += SR_THREADS) ys += __ldcg(yp + i);
+      for (int o = 16; o > 0; o >>= 1) ys += __shfl_xor_sync(0xffffffffu, ys, o);
+      if (lane == 0) sh.wsum[0][warp] = ys;
+      __syncthreads();
+      if (tid == 0) {
+        double s = 0;
+        for (int k = 0; k < 8; ++k) s += sh.wsum[0][k];
+        sh.s_sumy = s;
+      }
+      __syncthreads();
+    }
+    const double sumy = sh.s_sumy;
+    // sums of the vector blocks: warp sums, then one thread per block in warp order
+    auto block_sums = [&]() {
+      __syncthreads();
+      for (int vb = warp; vb < nvb; vb += 8)
+        if (lane == 0) {
+          double s = 0;
+          for (int k = 0; k < 8; ++k) s += sh.wsum[vb][k];
+          sh.vpart[vb] = s;
+        }
+      __syncthreads();
+    };
+    auto warp_put = [&](int vb, double s) {   // zero where the whole warp is past the end
+      if (vb * SR_THREADS + warp * 32 < Np)
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      if (lane == 0) sh.wsum[vb][warp] = s;
+    };
+    for (int vb = 0; vb < nvb; ++vb) {
+      const int t = vb * SR_THREADS + tid;
+      double s = 0;
+      if (t < Np) {
+        double acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+        int c = 0;
+        for (; c + 8 <= nch; c += 8)
+#pragma unroll
+          for (int u = 0; u < 8; ++u) acc[u] += __ldcg(part + (long long)(c + u) * Np + t);
+        for (; c < nch; ++c) acc[0] += __ldcg(part + (long long)c * Np + t);
+        const double a = ((acc[0] + acc[1]) + (acc[2] + acc[3])) + ((acc[4] + acc[5]) + (acc[6] + acc[7]));
+        const double qt = a - sumy * ob[t] + eps * p[t];
+        q[t] = qt;
+        s += p[t] * qt;
+      }
+      warp_put(vb, s);
+    }
+    block_sums();
+    if (warp == 0) {
+      const double pq = cgs_parts(sh.vpart, nvb, lane);
+      if (lane == 0) sh.s_alpha = sh.s_rr / pq;
+    }
+    __syncthreads();
+    // x, r, r.r
+    const double alpha = sh.s_alpha;
+    for (int vb = 0; vb < nvb; ++vb) {
+      const int t = vb * SR_THREADS + tid;
+      double s = 0;
+      if (t < Np) {
+        x[t] += alpha * p[t];
+        const double rt = r[t] - alpha * q[t];
+        r[t] = rt;
+        s += rt * rt;
+      }
+      warp_put(vb, s);
+    }
+    block_sums();
+    // beta from the tree sum; the stop test on the sum in block order
+    iters += 1;
+    if (warp == 0) {
+      const double rt = cgs_parts(sh.vpart, nvb, lane);
+      if (lane == 0) {
+        sh.s_beta = rt / sh.s_rr;
+        const double rr = sum_parts(sh.vpart, nvb);
+        sh.s_rr = rr;
+        if (iters >= maxit || !(sqrt(rr) > tol * gnorm)) sh.done = 1;
+      }
+    }
+    __syncthreads();
+    const double beta = sh.s_beta;
+    for (int vb = 0; vb < nvb; ++vb) {
+      const int t = vb * SR_THREADS + tid;
+      double s = 0;
+      if (t < Np) {
+        const double pt = r[t] + beta * p[t];
+        p[t] = pt;
+        s += ob[t] * pt;
+      }
+      warp_put(vb, s);
+    }
+    block_sums();
+  }
+  if (blockIdx.x == 0) {
+    for (int t = tid; t < Np; t += SR_THREADS) x_g[t] = x[t];
+    if (tid == 0) {
+      sc->rr = sh.s_rr;
+      sc->iters = iters;
+      sc->done = 1;
+    }
+  }
+}
+
 // theta -= tau x (and the float32 copy).
 __global__ void k_update(long long Np, double tau, const double* __restrict__ x,
                          double* __restrict__ theta, float* __restrict__ theta_f) {
