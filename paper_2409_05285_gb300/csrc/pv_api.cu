@@ -894,7 +894,7 @@ int init_runner_t(peps_ctx* c, int sms, BatchImpl<T>* b, int Dn, const T* theta,
   BatchBufs<T>::sizes(P->L1, P->L2, Dn, P->chi, sz, n8, nd);
   long long per = 0;
   for (long long x : sz) per += x;
-  size_t per_bytes = (size_t)per * sizeof(T) + (size_t)n8 + (size_t)nd * 8 + 16;
+  size_t per_bytes = (size_t)per * sizeof(T) + (size_t)n8 + (size_t)nd * 8 + 20;
   size_t fr = 0, tot = 0;
   cudaMemGetInfo(&fr, &tot);
   long long chunk = std::min<long long>({(long long)n, (long long)(fr / 2 / per_bytes), 65535LL});
@@ -908,6 +908,8 @@ int init_runner_t(peps_ctx* c, int sms, BatchImpl<T>* b, int Dn, const T* theta,
   if ((rc = dalloc(c, &i8, (size_t)n8 * chunk))) return rc;
   if ((rc = dalloc(c, &dbl, (size_t)nd * chunk * sizeof(double)))) return rc;
   if ((rc = dalloc(c, &b->es_tmp, (size_t)chunk * sizeof(double)))) return rc;
+  if ((rc = dalloc(c, &b->be.act_idx, (size_t)chunk * sizeof(int)))) return rc;
+  if ((rc = dalloc(c, &b->be.act_cnt, 2 * sizeof(int)))) return rc;
   if ((rc = dalloc(c, &b->d_sweep, sizeof(uint32_t)))) return rc;
   if (!c->d_jflops) {
     if ((rc = dalloc(c, &c->d_jflops, sizeof(double)))) return rc;

@@ -57,6 +57,14 @@ PV_HD Operand<T> batch_op(const T* base, long long stride) {
   return o;
 }
 
+// The chains an operation runs over: all n of them, or the *cnt listed ones.
+struct ChainList {
+  const int* idx = nullptr;
+  const int* cnt = nullptr;
+  PV_HD int count(int n) const { return cnt ? *cnt : n; }
+  PV_HD int chain(int k) const { return idx ? idx[k] : k; }
+};
+
 // Merged-dimension form of a contraction (as in contract()).
 struct MSpec {
   int no, nk;
@@ -704,6 +712,22 @@ struct BatchRunner {
   }
   static Operand<T> bat(const T* base, long long stride) { return batch_op<T>(base, stride); }
 
+  // Between guard_begin() and guard_end(), after sel(): operations whose results are read only for
+  // the chains that the proposal changes.  A back end without these runs them for every chain.
+  template <typename B>
+  static auto has_guard(B* p) -> decltype(p->guard_reset(), std::true_type());
+  static std::false_type has_guard(...);
+  static constexpr bool guards = decltype(has_guard((BE*)nullptr))::value;
+  void guard_reset() {
+    if constexpr (guards) be.guard_reset();
+  }
+  void guard_begin() {
+    if constexpr (guards) be.guard_begin();
+  }
+  void guard_end() {
+    if constexpr (guards) be.guard_end();
+  }
+
   void ein(T* out, long long os, const char* so, Operand<T> A, const char* sa, Operand<T> B,
            const char* sb, const Dims& d, int n, bool exact = false) {
     Spec raw = make_spec(so, sa, sb, d);
@@ -853,14 +877,29 @@ struct BatchRunner {
 
   // ----------------------------------------------------------------- strips
   // one-row strip pieces (U row = up env of row r, Dn row = down env r+1)
-  void s1_left(int r, int c, T* Lout, long long los, Operand<T> Lin, Operand<T> A, int n) {
+  // A step of a left partial in two parts: the product of the partial with the up environment,
+  // which does not depend on the site's local index, and the rest.  The proposals, the site
+  // environment and the advance of one column share the first part (pre1(), kept in the work
+  // buffer of the compression, which is idle during the strips): of 3 contractions a step,
+  // 1 is made once per column instead of 3 (sweep) or 4 (evaluation) times.
+  Operand<T> pre1() const { return bat(b.Cs, b.CB); }
+  void s1_pre(int r, int c, T* t, long long ts, Operand<T> Lin, int n) {
     const std::vector<int>&bu = shp.up[r], &bd = shp.down[r + 1];
     Dims dm;
-    dm.set('a', bu[c]).set('x', bu[c + 1]).set('b', bd[c]).set('y', bd[c + 1]);
+    dm.set('a', bu[c]).set('x', bu[c + 1]).set('b', bd[c]).set('l', dl(c)).set('u', du(r));
+    ein(t, ts, "lbux", Lin, "alb", envt(uprow(r), b.sU, c), "aux", dm, n);
+  }
+  void s1_post(int r, int c, T* Lout, long long los, Operand<T> t, Operand<T> A, int n) {
+    const std::vector<int>&bu = shp.up[r], &bd = shp.down[r + 1];
+    Dims dm;
+    dm.set('x', bu[c + 1]).set('b', bd[c]).set('y', bd[c + 1]);
     dm.set('l', dl(c)).set('r', dr(c)).set('u', du(r)).set('d', dd(r));
-    ein(b.t0, b.TMP, "lbux", Lin, "alb", envt(uprow(r), b.sU, c), "aux", dm, n);
-    ein(b.t1, b.TMP, "bxrd", bat(b.t0, b.TMP), "lbux", A, "lrud", dm, n);
+    ein(b.t1, b.TMP, "bxrd", t, "lbux", A, "lrud", dm, n);
     ein(Lout, los, "xry", bat(b.t1, b.TMP), "bxrd", envt(downrow(r + 1), b.sD, c), "bdy", dm, n);
+  }
+  void s1_left(int r, int c, T* Lout, long long los, Operand<T> Lin, Operand<T> A, int n) {
+    s1_pre(r, c, b.t0, b.TMP, Lin, n);
+    s1_post(r, c, Lout, los, bat(b.t0, b.TMP), A, n);
   }
   void s1_right(int r, int c, T* Rout, long long ros, Operand<T> Rin, Operand<T> A, int n) {
     const std::vector<int>&bu = shp.up[r], &bd = shp.down[r + 1];
@@ -872,27 +911,42 @@ struct BatchRunner {
     ein(Rout, ros, "alb", envt(uprow(r), b.sU, c), "aux", bat(b.t1, b.TMP), "lubx", dm, n);
   }
   void s1_env(int r, int c, Operand<T> L, Operand<T> R, int n) {
+    s1_pre(r, c, b.t0, b.TMP, L, n);
+    s1_env_post(r, c, bat(b.t0, b.TMP), R, n);
+  }
+  void s1_env_post(int r, int c, Operand<T> t, Operand<T> R, int n) {
     const std::vector<int>&bu = shp.up[r], &bd = shp.down[r + 1];
     Dims dm;
-    dm.set('a', bu[c]).set('x', bu[c + 1]).set('b', bd[c]).set('y', bd[c + 1]);
+    dm.set('x', bu[c + 1]).set('b', bd[c]).set('y', bd[c + 1]);
     dm.set('l', dl(c)).set('r', dr(c)).set('u', du(r)).set('d', dd(r));
-    ein(b.t0, b.TMP, "lbux", L, "alb", envt(uprow(r), b.sU, c), "aux", dm, n);
-    ein(b.t1, b.TMP, "lbury", bat(b.t0, b.TMP), "lbux", R, "xry", dm, n);
+    ein(b.t1, b.TMP, "lbury", t, "lbux", R, "xry", dm, n);
     ein(b.envo, b.D4, "lrud", bat(b.t1, b.TMP), "lbury", envt(downrow(r + 1), b.sD, c), "bdy", dm, n);
   }
   long long s1_len(int r, int c) const {
     return (long long)shp.up[r][c] * (c < L2 ? dl(c) : 1) * shp.down[r + 1][c];
   }
   // two-row strip pieces (U = up env of row r, rows r and r+1, Dn = down env r+2)
+  // (in two parts, as the one-row step)
+  void s2_pre(int r, int c, T* t, long long ts, Operand<T> Lin, int n) {
+    const std::vector<int>&bu = shp.up[r], &bd = shp.down[r + 2];
+    Dims dm;
+    dm.set('a', bu[c]).set('x', bu[c + 1]).set('b', bd[c]);
+    dm.set('i', dl(c)).set('j', dl(c)).set('u', du(r));
+    ein(t, ts, "ijbux", Lin, "aijb", envt(uprow(r), b.sU, c), "aux", dm, n);
+  }
   void s2_left(int r, int c, T* Lout, long long los, Operand<T> Lin, Operand<T> A1, Operand<T> A2,
+               int n) {
+    s2_pre(r, c, b.t0, b.TMP, Lin, n);
+    s2_post(r, c, Lout, los, bat(b.t0, b.TMP), A1, A2, n);
+  }
+  void s2_post(int r, int c, T* Lout, long long los, Operand<T> t, Operand<T> A1, Operand<T> A2,
                int n) {
     const std::vector<int>&bu = shp.up[r], &bd = shp.down[r + 2];
     Dims dm;
-    dm.set('a', bu[c]).set('x', bu[c + 1]).set('b', bd[c]).set('y', bd[c + 1]);
+    dm.set('x', bu[c + 1]).set('b', bd[c]).set('y', bd[c + 1]);
     dm.set('i', dl(c)).set('r', dr(c)).set('j', dl(c)).set('s', dr(c));
     dm.set('u', du(r)).set('m', dd(r)).set('d', dd(r + 1));
-    ein(b.t0, b.TMP, "ijbux", Lin, "aijb", envt(uprow(r), b.sU, c), "aux", dm, n);
-    ein(b.t1, b.TMP, "jbxrm", bat(b.t0, b.TMP), "ijbux", A1, "irum", dm, n);
+    ein(b.t1, b.TMP, "jbxrm", t, "ijbux", A1, "irum", dm, n);
     ein(b.t0, b.TMP, "bxrsd", bat(b.t1, b.TMP), "jbxrm", A2, "jsmd", dm, n);
     ein(Lout, los, "xrsy", bat(b.t0, b.TMP), "bxrsd", envt(downrow(r + 2), b.sD, c), "bdy", dm, n);
   }
@@ -919,6 +973,7 @@ struct BatchRunner {
   // ------------------------------------------------------------------- evaluation
   void eval(const uint8_t* S, int n, double* log_abs, int8_t* sign, double* es, double* ea,
             OT* O, long long No, bool cached) {
+    guard_reset();
     build_down(S, n);
     // diagonal energies
     be.diag(S, n, es, ea);
@@ -933,19 +988,22 @@ struct BatchRunner {
       T* Ln = b.p1L + b.P1;
       be.set(b.p1L, b.sp1L, 0, (T)1, n);
       for (int c = 0; c < L2; ++c) {
+        if (O || c + 1 < L2) s1_pre(r, c, b.Cs, b.CB, bat(Lc, b.sp1L), n);
         if (O) {
-          s1_env(r, c, bat(Lc, b.sp1L), bat(p1R(c + 1), b.sp1R), n);
+          s1_env_post(r, c, pre1(), bat(p1R(c + 1), b.sp1R), n);
           be.writeO(O, No, ooff[r * L2 + c], b.envo, b.D4, szs(r, c), b.p1R, b.sp1R, n);
         }
         if (c + 1 < L2) {
           for (int layer = 0; layer < 2; ++layer) {
             be.sel(ElemSel{S, N, r * L2 + c, r * L2 + c + 1, 1 + layer, b.si, b.sj, b.valid}, n);
-            s1_left(r, c, b.m0, b.P2, bat(Lc, b.sp1L), site_sel(r, c, b.si), n);
+            guard_begin();
+            s1_post(r, c, b.m0, b.P2, pre1(), site_sel(r, c, b.si), n);
             s1_left(r, c + 1, b.m1, b.P2, bat(b.m0, b.P2), site_sel(r, c + 1, b.sj), n);
             be.dot(OpDot<T>{b.m1, b.P2, p1R(c + 2), b.sp1R, s1_len(r, c + 2), b.num}, n);
+            guard_end();
             be.ratio(b.num, b.p1R, b.sp1R, b.valid, 0.5 * J1, layer == 0 ? es : ea, n);
           }
-          s1_left(r, c, Ln, b.sp1L, bat(Lc, b.sp1L), site(r, c, S), n);
+          s1_post(r, c, Ln, b.sp1L, pre1(), site(r, c, S), n);
           T* t = Lc;
           Lc = Ln;
           Ln = t;
@@ -960,10 +1018,13 @@ struct BatchRunner {
         be.set(b.p2L, b.sp2L, 0, (T)1, n);
         for (int c = 0; c < L2; ++c) {
           int i = r * L2 + c, j = i + L2;
+          s2_pre(r, c, b.Cs, b.CB, bat(L2c, b.sp2L), n);
           for (int layer = 0; layer < 2; ++layer) {
             be.sel(ElemSel{S, N, i, j, 1 + layer, b.si, b.sj, b.valid}, n);
-            s2_left(r, c, b.m0, b.P2, bat(L2c, b.sp2L), site_sel(r, c, b.si), site_sel(r + 1, c, b.sj), n);
+            guard_begin();
+            s2_post(r, c, b.m0, b.P2, pre1(), site_sel(r, c, b.si), site_sel(r + 1, c, b.sj), n);
             be.dot(OpDot<T>{b.m0, b.P2, p2R(c + 1), b.sp2R, s2_len(r, c + 1), b.num}, n);
+            guard_end();
             be.ratio(b.num, b.p2R, b.sp2R, b.valid, 0.5 * J1, layer == 0 ? es : ea, n);
           }
           if (J2 != 0.0 && c + 1 < L2) {
@@ -977,14 +1038,16 @@ struct BatchRunner {
                 Operand<T> s10 = diag == 0 ? site(r + 1, c, S) : site_sel(r + 1, c, b.sj);
                 Operand<T> s01 = diag == 0 ? site(r, c + 1, S) : site_sel(r, c + 1, b.si);
                 Operand<T> s11 = diag == 0 ? site_sel(r + 1, c + 1, b.sj) : site(r + 1, c + 1, S);
-                s2_left(r, c, b.m0, b.P2, bat(L2c, b.sp2L), s00, s10, n);
+                guard_begin();
+                s2_post(r, c, b.m0, b.P2, pre1(), s00, s10, n);
                 s2_left(r, c + 1, b.m1, b.P2, bat(b.m0, b.P2), s01, s11, n);
                 be.dot(OpDot<T>{b.m1, b.P2, p2R(c + 2), b.sp2R, s2_len(r, c + 2), b.num}, n);
+                guard_end();
                 be.ratio(b.num, b.p2R, b.sp2R, b.valid, 0.5 * J2, layer == 0 ? es : ea, n);
               }
             }
           }
-          s2_left(r, c, L2n, b.sp2L, bat(L2c, b.sp2L), site(r, c, S), site(r + 1, c, S), n);
+          s2_post(r, c, L2n, b.sp2L, pre1(), site(r, c, S), site(r + 1, c, S), n);
           T* t = L2c;
           L2c = L2n;
           L2n = t;
@@ -998,6 +1061,7 @@ struct BatchRunner {
   // -------------------------------------------------------------------- Metropolis
   void mc(uint8_t* S, int n, int p, uint64_t seed, int chain0, uint32_t sweep, int* acc,
           int* prop) {
+    guard_reset();
     build_down(S, n);
     trivial(uprow(0), b.sU, n);
     for (int r = 0; r < L1; ++r) {
@@ -1008,12 +1072,14 @@ struct BatchRunner {
       T* Ln = b.p1L + b.P1;
       be.set(b.p1L, b.sp1L, 0, (T)1, n);
       // P = Lc x column c at the current S (m0); X, Y proposals (m2, m3); Q = P x column c+1 (m1)
-      s1_left(r, 0, b.m0, b.P2, bat(Lc, b.sp1L), site(r, 0, S), n);
+      s1_pre(r, 0, b.Cs, b.CB, bat(Lc, b.sp1L), n);
+      s1_post(r, 0, b.m0, b.P2, pre1(), site(r, 0, S), n);
       for (int c = 0; c < L2; ++c) {
         int i = r * L2 + c;
+        if (c > 0) s1_pre(r, c, b.Cs, b.CB, bat(Lc, b.sp1L), n);
         be.dot(OpDot<T>{b.m0, b.P2, p1R(c + 1), b.sp1R, s1_len(r, c + 1), b.den}, n);
         be.sel(ElemSel{S, N, i, -1, 0, b.si, b.sj, b.valid}, n);
-        s1_left(r, c, b.m2, b.P2, bat(Lc, b.sp1L), site_sel(r, c, b.si), n);
+        s1_post(r, c, b.m2, b.P2, pre1(), site_sel(r, c, b.si), n);
         be.dot(OpDot<T>{b.m2, b.P2, p1R(c + 1), b.sp1R, s1_len(r, c + 1), b.num}, n);
         be.accept(ElemAccept<T>{S, N, i, -1, b.si, b.sj, b.valid, b.num, b.den, p, seed, chain0,
                                 sweep, (uint32_t)(8 * i), acc, prop, b.accepted, sweep_dev}, n);
@@ -1023,9 +1089,11 @@ struct BatchRunner {
           be.dot(OpDot<T>{b.m1, b.P2, p1R(c + 2), b.sp1R, s1_len(r, c + 2), b.den}, n);
           for (int layer = 0; layer < 2; ++layer) {
             be.sel(ElemSel{S, N, i, i + 1, 1 + layer, b.si, b.sj, b.valid}, n);
-            s1_left(r, c, b.m2, b.P2, bat(Lc, b.sp1L), site_sel(r, c, b.si), n);
+            guard_begin();
+            s1_post(r, c, b.m2, b.P2, pre1(), site_sel(r, c, b.si), n);
             s1_left(r, c + 1, b.m3, b.P2, bat(b.m2, b.P2), site_sel(r, c + 1, b.sj), n);
             be.dot(OpDot<T>{b.m3, b.P2, p1R(c + 2), b.sp1R, s1_len(r, c + 2), b.num}, n);
+            guard_end();
             be.accept(ElemAccept<T>{S, N, i, i + 1, b.si, b.sj, b.valid, b.num, b.den, p, seed,
                                     chain0, sweep, (uint32_t)(8 * i + 1 + layer), acc, prop,
                                     b.accepted, sweep_dev}, n);
@@ -1049,12 +1117,15 @@ struct BatchRunner {
         be.set(b.p2L, b.sp2L, 0, (T)1, n);
         for (int c = 0; c < L2; ++c) {
           int i = r * L2 + c, j = i + L2;
-          s2_left(r, c, b.m0, b.P2, bat(L2c, b.sp2L), site(r, c, S), site(r + 1, c, S), n);
+          s2_pre(r, c, b.Cs, b.CB, bat(L2c, b.sp2L), n);
+          s2_post(r, c, b.m0, b.P2, pre1(), site(r, c, S), site(r + 1, c, S), n);
           be.dot(OpDot<T>{b.m0, b.P2, p2R(c + 1), b.sp2R, s2_len(r, c + 1), b.den}, n);
           for (int layer = 0; layer < 2; ++layer) {
             be.sel(ElemSel{S, N, i, j, 1 + layer, b.si, b.sj, b.valid}, n);
-            s2_left(r, c, b.m1, b.P2, bat(L2c, b.sp2L), site_sel(r, c, b.si), site_sel(r + 1, c, b.sj), n);
+            guard_begin();
+            s2_post(r, c, b.m1, b.P2, pre1(), site_sel(r, c, b.si), site_sel(r + 1, c, b.sj), n);
             be.dot(OpDot<T>{b.m1, b.P2, p2R(c + 1), b.sp2R, s2_len(r, c + 1), b.num}, n);
+            guard_end();
             be.accept(ElemAccept<T>{S, N, i, j, b.si, b.sj, b.valid, b.num, b.den, p, seed, chain0,
                                     sweep, (uint32_t)(8 * i + 3 + layer), acc, prop, b.accepted, sweep_dev}, n);
             be.copy_masked(b.m0, b.P2, b.m1, b.P2, s2_len(r, c + 1), b.accepted, n);
@@ -1120,9 +1191,9 @@ constexpr int LQ_THREADS = 512;   // threads of the shared-memory Householder ke
 
 template <typename T>
 __global__ void __launch_bounds__(256) kb_ein(MSpec m, T* out, long long os, Operand<T> A,
-                                              Operand<T> B, int n, int quad) {
-  int s = blockIdx.y;
-  if (s >= n) return;
+                                              Operand<T> B, int n, int quad, ChainList cl) {
+  if ((int)blockIdx.y >= cl.count(n)) return;
+  const int s = cl.chain(blockIdx.y);
   const T* pa = A.at(s);
   const T* pb = B.at(s);
   T* po = out + (long long)s * os;
@@ -1143,7 +1214,7 @@ __global__ void __launch_bounds__(256) kb_ein(MSpec m, T* out, long long os, Ope
 template <typename T>
 __global__ void __launch_bounds__(256) kb_gemm(GSpec g, T* C, long long cs, Operand<T> A,
                                                Operand<T> B, int n, int TM, int TN, int KC,
-                                               int tilesN, int G) {
+                                               int tilesN, int G, ChainList cl) {
   extern __shared__ __align__(16) unsigned char dyn[];
   const int tid = threadIdx.x;
   const int tm = blockIdx.x / tilesN, tn = blockIdx.x % tilesN;
@@ -1173,10 +1244,11 @@ __global__ void __launch_bounds__(256) kb_gemm(GSpec g, T* C, long long cs, Oper
   const int per = (TM >> 2) * tnx;          // compute threads per sample
   const int slot = tid / per, loc = tid - slot * per;
   const int tx = loc % tnx, ty = loc / tnx;
+  n = cl.count(n);
   for (int sbase = blockIdx.y * G; sbase < n; sbase += gridDim.y * G) {
     const int ns = min(G, n - sbase);
-    const int s = sbase + slot;
     const bool comp = slot < ns;
+    const int s = comp ? cl.chain(sbase + slot) : 0;
     T acc[4][4];
 #pragma unroll
     for (int i = 0; i < 4; ++i)
@@ -1194,7 +1266,7 @@ __global__ void __launch_bounds__(256) kb_gemm(GSpec g, T* C, long long cs, Oper
           if (idx < totA) {
             int gs = idx / chunkA, r = idx - gs * chunkA;
             int kk = r / TM, mm = r - kk * TM, k = k0 + kk;
-            if (k < g.K && rowA[mm] >= 0) v[u] = A.at(sbase + gs)[rowA[mm] + kAo[k]];
+            if (k < g.K && rowA[mm] >= 0) v[u] = A.at(cl.chain(sbase + gs))[rowA[mm] + kAo[k]];
           }
         }
 #pragma unroll
@@ -1210,7 +1282,7 @@ __global__ void __launch_bounds__(256) kb_gemm(GSpec g, T* C, long long cs, Oper
           if (idx < totB) {
             int gs = idx / chunkB, r = idx - gs * chunkB;
             int kk = r / TN, nn = r - kk * TN, k = k0 + kk;
-            if (k < g.K && colB[nn] >= 0) v[u] = B.at(sbase + gs)[colB[nn] + kBo[k]];
+            if (k < g.K && colB[nn] >= 0) v[u] = B.at(cl.chain(sbase + gs))[colB[nn] + kBo[k]];
           }
         }
 #pragma unroll
@@ -1573,10 +1645,11 @@ __global__ void __launch_bounds__(BT) kb_norm(OpNorm<T> op, int n) {
 
 // One warp per sample.
 template <typename T>
-__global__ void __launch_bounds__(256) kb_dot(OpDot<T> op, int n) {
-  int s = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  int lane = threadIdx.x & 31;
-  if (s >= n) return;
+__global__ void __launch_bounds__(256) kb_dot(OpDot<T> op, int n, ChainList cl) {
+  const int k0 = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  const int lane = threadIdx.x & 31;
+  if (k0 >= cl.count(n)) return;
+  const int s = cl.chain(k0);
   const T* a = op.a + (long long)s * op.as;
   const T* b = op.b + (long long)s * op.bs;
   T acc = 0;
@@ -1589,6 +1662,24 @@ template <typename F>
 __global__ void kb_elem(F f, int n) {
   int s = blockIdx.x * blockDim.x + threadIdx.x;
   if (s < n) f(s);
+}
+
+// Proposal of a bond exchange, and the list of the chains that it changes (in any order: no
+// chain's arithmetic depends on the others).  `zero` is the counter of the next proposal: the
+// kernels that read its last value have ended.
+static __global__ void __launch_bounds__(128) kb_sel_list(ElemSel f, int n, int* idx, int* cnt, int* zero) {
+  const int s = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
+  bool v = false;
+  if (s < n) {
+    f(s);
+    v = f.valid[s] != 0;
+  }
+  if (s == 0) *zero = 0;
+  const unsigned m = __ballot_sync(0xffffffffu, v);
+  int base = 0;
+  if (lane == 0 && m) base = atomicAdd(cnt, __popc(m));
+  base = __shfl_sync(0xffffffffu, base, 0);
+  if (v) idx[base + __popc(m & ((1u << lane) - 1u))] = s;
 }
 
 template <typename T>
@@ -1693,6 +1784,14 @@ struct CudaBE {
   bool tc_split = false; // ... with every operand split into two TF32 parts (3xTF32)
   int tc_min_rows = 64;  // smallest larger free side sent to the tensor cores
   BatchTune tune;        // launch shapes (autotuned; results do not depend on them)
+  // Chains whose proposed exchange changes the configuration (about half): between guard_begin()
+  // and guard_end() contractions and dot products run over these alone.  The results of the
+  // others are read by nothing.
+  int* act_idx = nullptr;   // the list (room for every chain)
+  int* act_cnt = nullptr;   // two counters, taken in turn
+  int act_cur = 0;
+  int act_n = -1;           // the listed chains, read back while launches are profiled (-1: n)
+  ChainList act;
   int* tc_err = nullptr; // raised by a tensor-core kernel whose completion wait ran out
   void (*tc_form_override)(TcSpec&) = nullptr;   // test hook: restrict the operand forms
   KProf* prof = nullptr; // launch counter and optional per-kernel timing
@@ -1748,12 +1847,40 @@ struct CudaBE {
     return lim;
   }
 
+  int guard_op = -1;
+  void guard_reset() {
+    act_cur = 0;
+    if (!rec) cudaMemsetAsync(act_cnt, 0, 2 * sizeof(int), st);
+  }
+  void guard_begin() {
+    if (rec) {
+      guard_op = (int)rec->ops.size();
+      rec->add(PG_SKIP);
+      return;
+    }
+    act.idx = act_idx;
+    act.cnt = act_cnt + (act_cur ^ 1);   // the counter of the last proposal
+    if (prof && prof->on) {
+      cudaMemcpyAsync(&act_n, act.cnt, sizeof(int), cudaMemcpyDeviceToHost, st);
+      cudaStreamSynchronize(st);
+    }
+  }
+  void guard_end() {
+    if (rec) {
+      rec->ops[guard_op].g.i[0] = (int)rec->ops.size() - guard_op - 1;
+      return;
+    }
+    act = ChainList();
+    act_n = -1;
+  }
+
   static int gx(long long n, int t) { return (int)((n + t - 1) / t); }
   int gblocks(int n) const { return n < 8 * sms ? n : 8 * sms; }
 
   void ein(const Spec& raw, const MSpec& m, T* out, long long os, Operand<T> A, Operand<T> B,
            int n, bool exact = false) {
     GSpec gs = gemm_spec(raw);
+    const int nw = act_n < 0 ? n : act_n;   // chains the profile counts
     if (rec) {
       rec->bytes += ein_bytes(raw, A, B, 1);
       if constexpr (std::is_same<T, float>::value) {
@@ -1806,9 +1933,9 @@ struct CudaBE {
           gy = gy < 1 ? 1 : (gy > n ? n : gy);
           gy = gy > 65535 ? 65535 : gy;
           dim3 gr(tilesM * tilesN, (unsigned)gy);
-          PV_KLAUNCH(prof, st, "kb_gemm_tc2", ein_bytes(raw, A, B, n), 2.0 * raw.total * raw.kprod * n,
+          PV_KLAUNCH(prof, st, "kb_gemm_tc2", ein_bytes(raw, A, B, nw), 2.0 * raw.total * raw.kprod * nw,
                      kb_gemm_tc2<<<gr, TC_THREADS, bytes, st>>>(t, out, os, swap ? B : A, swap ? A : B, n,
-                                                                tilesN, tc_err));
+                                                                tilesN, tc_err, act));
           return;
         }
         // stay within the 200 KB of shared memory the kernel is configured for
@@ -1840,13 +1967,13 @@ struct CudaBE {
           gy = gy > 65535 ? 65535 : gy;
           dim3 gr(tilesM * tilesN, (unsigned)gy);
           if (t.pref)
-            PV_KLAUNCH(prof, st, "kb_gemm_tc", ein_bytes(raw, A, B, n), 2.0 * raw.total * raw.kprod * n,
+            PV_KLAUNCH(prof, st, "kb_gemm_tc", ein_bytes(raw, A, B, nw), 2.0 * raw.total * raw.kprod * nw,
                        kb_gemm_tc<true><<<gr, TC_THREADS, bytes, st>>>(t, out, os, swap ? B : A,
-                                                                       swap ? A : B, n, tilesN, tc_err));
+                                                                       swap ? A : B, n, tilesN, tc_err, act));
           else
-            PV_KLAUNCH(prof, st, "kb_gemm_tc", ein_bytes(raw, A, B, n), 2.0 * raw.total * raw.kprod * n,
+            PV_KLAUNCH(prof, st, "kb_gemm_tc", ein_bytes(raw, A, B, nw), 2.0 * raw.total * raw.kprod * nw,
                        kb_gemm_tc<false><<<gr, TC_THREADS, bytes, st>>>(t, out, os, swap ? B : A,
-                                                                        swap ? A : B, n, tilesN, tc_err));
+                                                                        swap ? A : B, n, tilesN, tc_err, act));
           return;
         }
       }
@@ -1871,15 +1998,15 @@ struct CudaBE {
       int gy = (n + G - 1) / G;
       if (gy > 65535) gy = 65535;
       dim3 gr(tilesN * tilesM, gy);
-      PV_KLAUNCH(prof, st, "kb_gemm", ein_bytes(raw, A, B, n), 2.0 * raw.total * raw.kprod * n,
-                 kb_gemm<T><<<gr, 256, bytes, st>>>(gs, out, os, A, B, n, TM, TN, KC, tilesN, G));
+      PV_KLAUNCH(prof, st, "kb_gemm", ein_bytes(raw, A, B, nw), 2.0 * raw.total * raw.kprod * nw,
+                 kb_gemm<T><<<gr, 256, bytes, st>>>(gs, out, os, A, B, n, TM, TN, KC, tilesN, G, act));
       return;
     }
     int quad = quad_ok(m) ? 1 : 0;
     long long work = quad ? (m.total >> 2) : m.total;
     dim3 g(gx(work, 256), n);
-    PV_KLAUNCH(prof, st, "kb_ein", ein_bytes(raw, A, B, n), 2.0 * raw.total * raw.kprod * n,
-               kb_ein<T><<<g, 256, 0, st>>>(m, out, os, A, B, n, quad));
+    PV_KLAUNCH(prof, st, "kb_ein", ein_bytes(raw, A, B, nw), 2.0 * raw.total * raw.kprod * nw,
+               kb_ein<T><<<g, 256, 0, st>>>(m, out, os, A, B, n, quad, act));
   }
   void lq(OpLq<T> op, int n) {
     const int K = op.m < op.nn ? op.m : op.nn;
@@ -2025,7 +2152,7 @@ struct CudaBE {
       o.g.l[2] = op.len;
       return;
     }
-    PV_KLAUNCH(prof, st, "kb_dot", 0.0, 0.0, kb_dot<T><<<gx(n, 8), 256, 0, st>>>(op, n));
+    PV_KLAUNCH(prof, st, "kb_dot", 0.0, 0.0, kb_dot<T><<<gx(n, 8), 256, 0, st>>>(op, n, act));
   }
   void set(T* x, long long xs, long long off, T v, int n) {
     if (rec) {
@@ -2127,7 +2254,13 @@ struct CudaBE {
       o.g.i[2] = f.kind;
       return;
     }
-    PV_KLAUNCH(prof, st, "kb_elem_sel", 0.0, 0.0, kb_elem<<<gx(n, 128), 128, 0, st>>>(f, n));
+    if (f.kind == 0) {   // a flip changes every chain
+      PV_KLAUNCH(prof, st, "kb_elem_sel", 0.0, 0.0, kb_elem<<<gx(n, 128), 128, 0, st>>>(f, n));
+      return;
+    }
+    PV_KLAUNCH(prof, st, "kb_elem_sel", 0.0, 0.0,
+               kb_sel_list<<<gx(n, 128), 128, 0, st>>>(f, n, act_idx, act_cnt + act_cur, act_cnt + (act_cur ^ 1)));
+    act_cur ^= 1;
   }
   void ratio(const T* num, const T* den, long long dens, const int8_t* valid, double coef,
              double* e, int n) {

@@ -117,13 +117,14 @@ void direct_rows(BatchRunner<T, BE, OT>& run, uint8_t* S, int n, const double* u
     be.set(b.p1L, b.sp1L, 0, (T)1, n);
     for (int c = 0; c < L2; ++c) {
       const int i = r * L2 + c;
+      run.s1_pre(r, c, b.Cs, b.CB, run.bat(Lc, b.sp1L), n);
       for (int s = 0; s < 4; ++s) {
         be.set_i8(b.si, (int8_t)s, n);
-        run.s1_left(r, c, b.m2, b.P2, run.bat(Lc, b.sp1L), run.site_sel(r, c, b.si), n);
+        run.s1_post(r, c, b.m2, b.P2, run.pre1(), run.site_sel(r, c, b.si), n);
         be.dot(OpDot<T>{b.m2, b.P2, run.p1R(c + 1), b.sp1R, run.s1_len(r, c + 1), cand[s]}, n);
       }
       be.draw(ElemDraw<T>{S, N, i, cand[0], cand[1], cand[2], cand[3], b_d, expo, u, logq}, n);
-      run.s1_left(r, c, Ln, b.sp1L, run.bat(Lc, b.sp1L), run.site(r, c, S), n);
+      run.s1_post(r, c, Ln, b.sp1L, run.pre1(), run.site(r, c, S), n);
       T* t = Lc;
       Lc = Ln;
       Ln = t;

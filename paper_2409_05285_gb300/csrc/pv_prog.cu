@@ -598,6 +598,7 @@ __global__ void __launch_bounds__(512, 1) kb_prog(const PgOp* __restrict__ ops, 
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
   bool stop = false;
+  int skip = 0;   // operations still to leave out (the same in every thread)
   for (int s = blockIdx.x; s < a.n && !stop; s += gridDim.x) {
     const uint8_t* S = (const uint8_t*)a.slot[PS_S] + (long long)s * a.N;
     for (int i = tid; i < a.N; i += nthr) sh.S[i] = S[i];
@@ -609,10 +610,15 @@ __global__ void __launch_bounds__(512, 1) kb_prog(const PgOp* __restrict__ ops, 
       for (int q = 0; q < PG_BLOCK; ++q) {
         const PgOp& o = sh.op[b & 1][q];
         if (o.kind < 0) break;
+        if (skip > 0) {
+          --skip;
+          continue;
+        }
         if (o.kind >= PG_T0) {
           if (warp == 0) pg_op0<T>(b & 1, q, s, a);
         } else {
           switch (o.kind) {
+            case PG_SKIP: skip = sh.i8[2] ? 0 : o.g.i[0]; break;
             case PG_FMA: pg_do_fma<T>(b & 1, q, s, a, tab); break;
             case PG_TC:
               if constexpr (sizeof(T) == 4) pg_do_tc(b & 1, q, s, a, tab, ts);

@@ -30,6 +30,7 @@ namespace pv {
 
 enum PgKind : int {
   PG_FMA, PG_TC, PG_EIN, PG_COPY, PG_NORM, PG_LQ, PG_LQ2, PG_CHOL, PG_TRUNC, PG_TRUNC64, PG_O, PG_DIAG,
+  PG_SKIP,   // the next i[0] operations are left out where the proposal changes nothing
   // executed by the first thread (PG_DOT: the first warp): no barrier between two of them
   PG_T0, PG_SET = PG_T0, PG_SETD, PG_COPYD, PG_SETI8, PG_SEL, PG_DOT, PG_RATIO, PG_ACCEPT, PG_AMP, PG_DRAW
 };

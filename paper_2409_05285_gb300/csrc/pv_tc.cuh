@@ -481,7 +481,7 @@ __device__ __forceinline__ void tc_epilogue(const TcSpec& t, uint32_t tmem, floa
 template <bool PREF>
 __global__ void __launch_bounds__(TC_THREADS) kb_gemm_tc(TcSpec t, float* C, long long cs,
                                                          Operand<float> P, Operand<float> Q,
-                                                         int n, int tilesN, int* err) {
+                                                         int n, int tilesN, int* err, ChainList cl) {
   extern __shared__ __align__(16) unsigned char dyn[];
   __shared__ __align__(8) uint64_t bar[2];
   __shared__ uint32_t tslot;
@@ -538,6 +538,7 @@ __global__ void __launch_bounds__(TC_THREADS) kb_gemm_tc(TcSpec t, float* C, lon
   const uint32_t tmem = tslot;
   const uint32_t idesc = tc_idesc(TC_ROWS, TN);
   const int Kp = ((t.K + 7) >> 3) << 3;
+  n = cl.count(n);
   uint32_t ph = 0u;   // phase bits of the two barriers (bit i: barrier i)
 
   if (nst == 2) {
@@ -546,14 +547,16 @@ __global__ void __launch_bounds__(TC_THREADS) kb_gemm_tc(TcSpec t, float* C, lon
     // their prefetched registers are stored), and chain i's epilogue follows the next MMA.
     float4 ra[PREF ? 4 : 1], rb[PREF ? 2 : 1];
     int it = 0, prev = -1;
-    int s = blockIdx.y;
+    int k = blockIdx.y;
     if constexpr (PREF) {
-      if (s < n) {
+      if (k < n) {
+        const int s = cl.chain(k);
         tc_pload(ra, P.at(s), t.modeP, rowsA, Kc, t.K, rowP, kPo, tid);
         if (!t.sym) tc_pload(rb, Q.at(s), t.modeQ, rowsB, Kc, t.K, colQ, kQo, tid);
       }
     }
-    for (; s < n; s += gridDim.y, ++it) {
+    for (; k < n; k += gridDim.y, ++it) {
+      const int s = cl.chain(k);
       const int st = it & 1;
       float* As = stage0 + (long long)st * sst;
       float* Bs = t.sym ? As : As + sa;
@@ -579,8 +582,8 @@ __global__ void __launch_bounds__(TC_THREADS) kb_gemm_tc(TcSpec t, float* C, lon
         tc_commit(st ? bar1 : bar0);
       }
       if constexpr (PREF) {
-        const int sn = s + gridDim.y;
-        if (sn < n) {
+        if (k + (int)gridDim.y < n) {
+          const int sn = cl.chain(k + gridDim.y);
           tc_pload(ra, P.at(sn), t.modeP, rowsA, Kc, t.K, rowP, kPo, tid);
           if (!t.sym) tc_pload(rb, Q.at(sn), t.modeQ, rowsB, Kc, t.K, colQ, kQo, tid);
         }
@@ -627,7 +630,8 @@ __global__ void __launch_bounds__(TC_THREADS) kb_gemm_tc(TcSpec t, float* C, lon
     const uint32_t a = tc_smem_addr(As), b = tc_smem_addr(Bs);
     const uint32_t al = t.split ? tc_smem_addr(Al) : 0, bl = t.split ? tc_smem_addr(Bl) : 0;
     bool ok = true;
-    for (int s = blockIdx.y; s < n && ok; s += gridDim.y) {
+    for (int k = blockIdx.y; k < n && ok; k += gridDim.y) {
+      const int s = cl.chain(k);
       const float* pp = P.at(s);
       const float* pq = Q.at(s);
       for (int k0 = 0; k0 < t.K; k0 += Kc) {

@@ -133,7 +133,7 @@ __device__ __forceinline__ void tc2_chunk(float* dst, float* dlo, const float* _
 
 static __global__ void __launch_bounds__(TC_THREADS) kb_gemm_tc2(TcSpec t, float* C, long long cs,
                                                           Operand<float> P, Operand<float> Q, int n,
-                                                          int tilesN, int* err) {
+                                                          int tilesN, int* err, ChainList cl) {
   extern __shared__ __align__(16) unsigned char dyn[];
   __shared__ __align__(8) uint64_t mbar[TC2_MAXST];
   __shared__ uint32_t tslot;
@@ -187,6 +187,7 @@ static __global__ void __launch_bounds__(TC_THREADS) kb_gemm_tc2(TcSpec t, float
   const int Kp = ((t.K + 7) >> 3) << 3;
   const int nk = (t.K + Kc - 1) / Kc;
   const int gy = gridDim.y;
+  n = cl.count(n);
   const int nch = blockIdx.y < n ? (n - 1 - blockIdx.y) / gy + 1 : 0;
   const long long total = (long long)nch * nk;
 
@@ -194,7 +195,7 @@ static __global__ void __launch_bounds__(TC_THREADS) kb_gemm_tc2(TcSpec t, float
   // copies (round = false) or rounding (round = true) of item j's operand chunks
   auto chunk = [&](long long j, bool round) {
     const int c = (int)(j / nk), kc = (int)(j - (long long)c * nk);
-    const int s = blockIdx.y + c * gy;
+    const int s = cl.chain(blockIdx.y + c * gy);
     float* As = stA(j);
     float* Bs = t.sym ? As : As + sa;
     float* Al = t.split ? As + sa + sb : nullptr;
@@ -213,7 +214,7 @@ static __global__ void __launch_bounds__(TC_THREADS) kb_gemm_tc2(TcSpec t, float
   };
   auto epilogue = [&](long long j) {   // chain of item j, accumulator of that chain
     const int c = (int)(j / nk);
-    const int s = blockIdx.y + c * gy;
+    const int s = cl.chain(blockIdx.y + c * gy);
     tc_fence_after();
     tc_epilogue(t, tmem + (uint32_t)((c % nacc) * TN), C + (long long)s * cs, rowC, colC, warp, lane);
     tc_fence_before();
