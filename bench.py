@@ -78,7 +78,7 @@ NCU_TRAFFIC = {
                   "step at 512 chains (default shapes, no autotune), scaled by algorithmic bytes",
     },
 }
-TRAFFIC_SOURCES = ("paper_2409_05285_gb300/csrc/pv_tc.cuh", "paper_2409_05285_gb300/csrc/pv_tc2.cuh",
+TRAFFIC_SOURCES = ("paper_2409_05285_gb300/csrc/pv_tc.cuh", "paper_2409_05285_gb300/csrc/pv_gemm.cuh",
                    "paper_2409_05285_gb300/csrc/pv_batch.cuh")
 
 
@@ -228,7 +228,7 @@ def tf32_peak(peaks):
 def kernel_roofline(kstats, peaks, prec, binding):
     """Roofline of the dominant kernel from the library's per-launch CUDA events (taken on an
     untimed step): achieved = algorithmic flops (tensor-core contractions) or bytes per launch /
-    mean launch time.  The tensor-core contractions (register-staged and cp.async-pipelined)
+    mean launch time.  The tensor-core contractions
     are bounded by the tensor pipe (TF32 peak); their HBM view (algorithmic bytes / time
     against the measured copy bandwidth) is given too."""
     total = sum(v[1] for v in kstats.values()) or 1.0
@@ -241,7 +241,7 @@ def kernel_roofline(kstats, peaks, prec, binding):
     name, (n, ms, nbytes, flops) = max(kstats.items(), key=lambda kv: kv[1][1])
     hbm = peaks.get("hbm_gbs")
     hpeak, hsrc = (hbm, "measured") if hbm else (6800.0, "fallback")
-    if name in ("kb_gemm_tc", "kb_gemm_tc2") and flops > 0:
+    if name == "kb_gemm_tc" and flops > 0:
         peak, src = tf32_peak(peaks)
         achieved = flops / n / (ms / n / 1e3) / 1e12
         out = {"kernel": name, "bound": "tensor", "achieved": achieved, "peak": peak,

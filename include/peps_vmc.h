@@ -380,15 +380,13 @@ long long peps_launches(const peps_ctx* ctx);
  * context without the batched engine. */
 typedef struct {
   int grid_pct;    /* persistent tensor-core grid, per cent of the resident CTAs */
-  int db_bytes;    /* largest operand stage that is double-buffered */
+  int db_bytes;    /* kept for saved shapes; no effect */
   int ffma_g;      /* most chains per block of the FFMA contraction kernel */
   int kc_max;      /* largest contraction chunk of the tensor-core kernel (8, 16, ..., 64) */
   double ms_before, ms_after;
-  int pipelined;   /* contractions with vector operands on the cp.async-pipelined tensor-core
-                      kernel: 1 the short ones (K <= 64), 2 all; 0: every contraction takes
-                      the register-staged kernel */
-  int stage_kb;    /* shared memory of the pipelined kernel's stage ring per CTA, KB (32..200;
-                      0 in peps_set_tune keeps the current value) */
+  int pipelined;   /* kept for saved shapes; no effect */
+  int stage_kb;    /* kept for saved shapes; no effect (32..200; 0 in peps_set_tune keeps the
+                      current value) */
   int trunc_threads; /* threads of a Jacobi truncation block whose matrix fits in shared
                         memory: 32, 128 or 256, or 64 (the default) for the kernel's own choice
                         by the size and number of the matrices (0 in peps_set_tune keeps the

@@ -968,12 +968,12 @@ int init_runner_t(peps_ctx* c, int sms, BatchImpl<T>* b, int Dn, const T* theta,
     // also takes the right factors from the Gram matrix
     if ((rc = dalloc(c, &b->be.tc_err, sizeof(int)))) return rc;
     cudaError_t e = cudaMemsetAsync(b->be.tc_err, 0, sizeof(int), c->stream);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(kb_gemm_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(kb_gemm_tc2, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(kb_gemm_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    auto big = [&](auto k) {
+      if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    };
+    big(kb_gemm_tc<8, 4, 4>);
+    big(kb_gemm_tc<4, 4, 5>);
+    big(kb_gemm_tc<4, 8, 4>);
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(kb_chol<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     if (e != cudaSuccess) return fail(c, PEPS_ECUDA, std::string("tensor-core setup: ") + cudaGetErrorString(e));
@@ -1839,13 +1839,10 @@ int peps_autotune(peps_ctx* c, int reps, peps_tune* out) {
     PV_TRY(timed(&before));
     cur = before;
     // coordinate descent over the launch-shape parameters (results are the same for all)
-    const int grid_c[] = {50, 100, 200}, db_c[] = {0, 12 * 1024, 48 * 1024}, kc_c[] = {16, 32, 64},
-              p_c[] = {0, 1, 2}, sb_c[] = {64 * 1024, 96 * 1024, 192 * 1024}, g_c[] = {1, 16, 256},
-              tt_c[] = {32, 64, 256};
-    int* fields[] = {&tu.grid_pct, &tu.db_bytes, &tu.kc_max, &tu.pipelined, &tu.stage_budget, &tu.ffma_g,
-                     &tu.trunc_threads};
-    const int* cands[] = {grid_c, db_c, kc_c, p_c, sb_c, g_c, tt_c};
-    for (int knob = c->batch->uses_tensor_cores() ? 0 : 5; knob < 7; ++knob) {
+    const int grid_c[] = {50, 100, 200}, kc_c[] = {16, 32, 64}, g_c[] = {1, 16, 256}, tt_c[] = {32, 64, 256};
+    int* fields[] = {&tu.grid_pct, &tu.kc_max, &tu.ffma_g, &tu.trunc_threads};
+    const int* cands[] = {grid_c, kc_c, g_c, tt_c};
+    for (int knob = c->batch->uses_tensor_cores() ? 0 : 2; knob < 4; ++knob) {
       int* field = fields[knob];
       const int* cand = cands[knob];
       int best_v = *field;

@@ -9,6 +9,7 @@
 // Bond dimensions depend only on the position, so all shapes are known on the host.
 #pragma once
 
+#include <algorithm>
 #include <cstdint>
 #include <cmath>
 #include <vector>
@@ -1178,7 +1179,7 @@ inline void bond_lists(int L1, int L2, double J1, double J2, std::vector<int>& b
 }  // namespace pv
 
 #include "pv_tc.cuh"
-#include "pv_tc2.cuh"
+#include "pv_gemm.cuh"
 
 #if defined(__CUDACC__)
 #include "pv_prof.cuh"
@@ -1731,12 +1732,10 @@ constexpr int FFMA_K_MAX = 8192;
 // changes any result (each chain's arithmetic is the same in every choice).
 struct BatchTune {
   int grid_pct = 100;          // persistent tensor-core grid, per cent of the resident CTAs
-  int db_bytes = 12 * 1024;    // largest operand stage that gets two stages
   int ffma_g = 256;            // most chains per block of the FFMA GEMM
   int kc_max = 64;             // largest contraction chunk of the tensor-core GEMM
-  int pipelined = 1;           // tensor-core GEMM on the cp.async pipeline (kb_gemm_tc2): 0 none,
-                               // 1 short vector contractions (K <= 64), 2 every vector one
-  int stage_budget = 96 * 1024;   // ... bytes of copy stages per CTA
+  // of kernels that are gone; accepted and reported for callers that keep saved shapes
+  int db_bytes = 12 * 1024, pipelined = 1, stage_budget = 96 * 1024;
   int trunc_threads = 64;      // threads of a Jacobi truncation block (32, 128, 256) when its
                                // matrix is in shared memory (the same bits for each); 64: by
                                // the size and number of the matrices (jac_launch)
@@ -1814,39 +1813,6 @@ struct CudaBE {
     return (a * (A.mode == OP_BATCH ? n : sites) + b * (B.mode == OP_BATCH ? n : sites) + c * n) *
            sizeof(T);
   }
-  int tc2_regs = 0;
-  int tc2_reg_limit() {
-    if (!tc2_regs) {
-      cudaFuncAttributes fa;
-      int regs = 64;
-      if (cudaFuncGetAttributes(&fa, kb_gemm_tc2) == cudaSuccess && fa.numRegs > 0) regs = fa.numRegs;
-      else cudaGetLastError();
-      regs = (regs + 7) & ~7;
-      int lim = 65536 / (regs * TC_THREADS);
-      lim = lim > 2048 / TC_THREADS ? 2048 / TC_THREADS : lim;
-      tc2_regs = lim < 1 ? 1 : lim;
-    }
-    return tc2_regs;
-  }
-  // resident tensor-core GEMM CTAs per SM allowed by registers and threads (cached)
-  int tc_by_regs[2] = {0, 0};
-  int tc_reg_limit(bool pref) {
-    int& lim = tc_by_regs[pref ? 1 : 0];
-    if (!lim) {
-      cudaFuncAttributes fa;
-      int regs = 64;
-      cudaError_t e = pref ? cudaFuncGetAttributes(&fa, kb_gemm_tc<true>)
-                           : cudaFuncGetAttributes(&fa, kb_gemm_tc<false>);
-      if (e == cudaSuccess && fa.numRegs > 0) regs = fa.numRegs;
-      else cudaGetLastError();
-      regs = (regs + 7) & ~7;   // per-warp allocation granularity
-      lim = 65536 / (regs * TC_THREADS);
-      if (lim > 2048 / TC_THREADS) lim = 2048 / TC_THREADS;
-      if (lim < 1) lim = 1;
-    }
-    return lim;
-  }
-
   int guard_op = -1;
   void guard_reset() {
     act_cur = 0;
@@ -1907,73 +1873,25 @@ struct CudaBE {
         t.split = (exact || tc_split) ? 1 : 0;   // float32-accurate products (3xTF32)
         if (tc_form_override) tc_form_override(t);
         t.sym = tc_symmetric(t, op_same(A, B)) ? 1 : 0;
-        if (t.Kc > tune.kc_max) {   // smaller chunks: smaller stages, more resident CTAs
-          t.Kc = tune.kc_max;
-          if (t.K > t.Kc) t.pref = 0;
-        }
-        // the pipelined kernel wins (measured at the 10x10 D=6 chi=36 shapes) on short
-        // contractions (K <= 64) whose operands are both vector copies, and on those of at most
-        // 8 indices; element-wise gathers, long and split contractions stay on the
-        // register-staged kernel
-        const bool vec = t.modeP != TC_SCALAR && t.modeQ != TC_SCALAR;
-        if (tune.pipelined && ((vec && !t.split && (t.K <= 64 || tune.pipelined == 2)) || t.K <= 8)) {
-          // pipelined kernel: cp.async ring of stages over (chain, contraction chunk) items
-          if (t.Kc > tune.kc_max) t.Kc = tune.kc_max;
-          tc2_shape(t, (size_t)tune.stage_budget);
-          const int tilesM = (t.M + TC_ROWS - 1) / TC_ROWS, tilesN = (t.N + t.TN - 1) / t.TN;
-          const size_t bytes = tc2_smem_bytes(t);
-          int per_sm = (int)((size_t)(227 * 1024) / (bytes + 1024));
-          const int by_tmem = 512 / tc_cols(t.TN * t.nacc);
-          const int by_regs = tc2_reg_limit();
-          per_sm = per_sm < by_tmem ? per_sm : by_tmem;
-          per_sm = per_sm < by_regs ? per_sm : by_regs;
-          per_sm = per_sm < 16 ? per_sm : 16;
-          per_sm = per_sm < 1 ? 1 : per_sm;
-          long long gy = (long long)sms * per_sm * tune.grid_pct / (100LL * tilesM * tilesN);
-          gy = gy < 1 ? 1 : (gy > n ? n : gy);
-          gy = gy > 65535 ? 65535 : gy;
-          dim3 gr(tilesM * tilesN, (unsigned)gy);
-          PV_KLAUNCH(prof, st, "kb_gemm_tc2", ein_bytes(raw, A, B, nw), 2.0 * raw.total * raw.kprod * nw,
-                     kb_gemm_tc2<<<gr, TC_THREADS, bytes, st>>>(t, out, os, swap ? B : A, swap ? A : B, n,
-                                                                tilesN, tc_err, act));
-          return;
-        }
-        // stay within the 200 KB of shared memory the kernel is configured for
-        const size_t smem_cap = 200 * 1024;
-        while (tc_smem_bytes(t) > smem_cap && t.Kc > 8) {
-          t.Kc -= 8;
-          t.pref = 0;
-        }
-        {
-          // two operand stages and accumulators (consecutive chains pipelined) only for small
-          // single-chunk stages: larger ones cost more in resident CTAs than they gain
-          t.nst = (t.K <= t.Kc && tc_stage_bytes(t) <= (size_t)tune.db_bytes) ? 2 : 1;
-          if (tc_smem_bytes(t) > smem_cap) t.nst = 1;
-        }
-        if (tc_smem_bytes(t) <= smem_cap) {
-          const int tilesM = (t.M + TC_ROWS - 1) / TC_ROWS, tilesN = (t.N + t.TN - 1) / t.TN;
-          const size_t bytes = tc_smem_bytes(t);
-          // persistent grid of the CTAs that can be resident at once (shared memory, tensor
-          // memory columns, registers)
-          int per_sm = (int)((size_t)(227 * 1024) / (bytes + 1024));
-          int by_tmem = 512 / tc_cols(t.TN * tc_stages(t));
-          int by_regs = tc_reg_limit(t.pref != 0);
-          per_sm = per_sm < by_tmem ? per_sm : by_tmem;
-          per_sm = per_sm < by_regs ? per_sm : by_regs;
-          per_sm = per_sm < 16 ? per_sm : 16;
-          per_sm = per_sm < 1 ? 1 : per_sm;
-          long long gy = (long long)sms * per_sm * tune.grid_pct / (100LL * tilesM * tilesN);
-          gy = gy < 1 ? 1 : (gy > n ? n : gy);
-          gy = gy > 65535 ? 65535 : gy;
-          dim3 gr(tilesM * tilesN, (unsigned)gy);
-          if (t.pref)
+        tc_shape(t, tune.kc_max);
+        const size_t bytes = tc_smem_bytes(t);
+        if (bytes <= 200 * 1024) {   // what the kernels are configured for
+          // persistent grid of the CTAs that can be resident at once
+          auto go = [&](auto kern, int by_regs) {
+            const int tilesM = (t.M + TC_ROWS - 1) / TC_ROWS, tilesN = (t.N + t.TN - 1) / t.TN;
+            int per_sm = std::min((int)((size_t)(227 * 1024) / (bytes + 1024)), std::min(512 / tc_cols(t.TN), by_regs));
+            per_sm = per_sm < 1 ? 1 : per_sm;
+            long long gy = (long long)sms * per_sm * tune.grid_pct / (100LL * tilesM * tilesN);
+            gy = gy < 1 ? 1 : (gy > n ? n : gy);
+            gy = gy > 65535 ? 65535 : gy;
+            dim3 gr(tilesM * tilesN, (unsigned)gy);
             PV_KLAUNCH(prof, st, "kb_gemm_tc", ein_bytes(raw, A, B, nw), 2.0 * raw.total * raw.kprod * nw,
-                       kb_gemm_tc<true><<<gr, TC_THREADS, bytes, st>>>(t, out, os, swap ? B : A,
-                                                                       swap ? A : B, n, tilesN, tc_err, act));
-          else
-            PV_KLAUNCH(prof, st, "kb_gemm_tc", ein_bytes(raw, A, B, nw), 2.0 * raw.total * raw.kprod * nw,
-                       kb_gemm_tc<false><<<gr, TC_THREADS, bytes, st>>>(t, out, os, swap ? B : A,
-                                                                        swap ? A : B, n, tilesN, tc_err, act));
+                       kern<<<gr, TC_THREADS, bytes, st>>>(t, out, os, swap ? B : A, swap ? A : B, n, tilesN, tc_err,
+                                                           act));
+          };
+          if (t.Kc == 32) go(kb_gemm_tc<8, 4, 4>, 4);
+          else if (t.TN <= 128) go(kb_gemm_tc<4, 4, 5>, 5);
+          else go(kb_gemm_tc<4, 8, 4>, 4);
           return;
         }
       }
