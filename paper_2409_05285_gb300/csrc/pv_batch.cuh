@@ -1905,6 +1905,11 @@ struct CudaBE {
       if (Mp < TM) TM = Mp;
       int G = 256 / ((TM / 4) * (TN / 4));   // samples per block when one tile is small
       if (G > tune.ffma_g) G = tune.ffma_g;
+      // a block's time is its chunks' gather latency, whatever it holds: enough blocks for four
+      // per SM come first (192 chains: 12 blocks of 16 chains otherwise)
+      const int tiles = ((gs.N + TN - 1) / TN) * ((gs.M + TM - 1) / TM);
+      const long long gmax = (long long)n * tiles / (4LL * sms);
+      if (G > gmax) G = (int)gmax;
       if (G < 1) G = 1;
       int budget = (int)(6144 * 4 / sizeof(T));   // 24 KB of operand tiles
       int KC = budget / (G * (TM + TN));
