@@ -1567,11 +1567,18 @@ __device__ __forceinline__ void chol64(const OpChol<T>& op, int s, T* lc, T* red
 #pragma unroll
       for (int r = 0; r < R; ++r)
 #pragma unroll
-        for (int c = 0; c < 4; ++c)
-          if (c >= cj) a[r][c] -= li[r] * lk[c];
+        for (int c = 0; c < 4; ++c)   // entries of later columns, on and below the diagonal's 16 x TY blocks
+          if (c >= cj && TY * r + TY > 16 * c) a[r][c] -= li[r] * lk[c];
     }
   }
   __syncthreads();
+}
+
+template <typename T>
+__global__ void __launch_bounds__(128, 6) kb_chol64(OpChol<T> op, int n) {
+  __shared__ T lc[128];
+  __shared__ T red[32];
+  for (int s = blockIdx.x; s < n; s += gridDim.x) chol64<T, 8>(op, s, lc, red);
 }
 
 template <typename T, int NT = BT>
@@ -1580,8 +1587,7 @@ __global__ void __launch_bounds__(NT) kb_chol(OpChol<T> op, int n) {
   __shared__ T red[32];
   __shared__ T s_piv[2];
   for (int s = blockIdx.x; s < n; s += gridDim.x) {
-    if (NT == 256 && op.m <= 64) chol64<T, 16>(op, s, (T*)dyn, red);
-    else chol_matrix(op, s, (T*)dyn, red, s_piv);
+    chol_matrix(op, s, (T*)dyn, red, s_piv);
   }
 }
 
@@ -2038,6 +2044,12 @@ struct CudaBE {
       o.g.l[0] = op.gs;
       o.g.l[1] = op.ls;
       o.g.i[0] = op.m;
+      return;
+    }
+    if (op.m <= 64) {
+      const int grid = n < 6 * sms ? n : 6 * sms;   // resident at once
+      PV_KLAUNCH(prof, st, "kb_chol", (double)n * 2.0 * op.m * op.m * sizeof(T),
+                 (double)op.m * op.m * op.m / 3.0 * n, (kb_chol64<T><<<grid, 128, 0, st>>>(op, n)));
       return;
     }
     if (bytes > 96 * 1024 && (int)bytes <= chol_wide_max) {
