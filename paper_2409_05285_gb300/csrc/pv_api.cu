@@ -2178,6 +2178,7 @@ struct peps_famp {
   std::vector<long long> toff16, toff32;
   long long n16 = 0;
   int n_max = 0;
+  int piece = 0;           // configurations taken through the engine at a time (at least n_max)
   long long *d_toff16 = nullptr, *d_toff32 = nullptr;
   double* d_th16 = nullptr;
   void* d_th32 = nullptr;
@@ -2228,16 +2229,16 @@ struct peps_famp {
 namespace {
 
 // log|psi| and sign of `count` configurations already on the device (entries checked unless
-// `check` is off: the caller knows them valid): in pieces of n_max through the extended
-// indices and the engine.
+// `check` is off: the caller knows them valid): in pieces through the extended indices and the
+// engine.
 int famp_amplitudes(peps_famp* f, const uint8_t* dS, long long count, double* la, int8_t* sg,
                     bool check = true) {
   peps_ctx* c = f->c;
   const int N = c->N;
   cudaStream_t st = c->stream;
   if (check) PV_CUDA(c, cudaMemsetAsync(f->d_bad, 0, sizeof(int), st));
-  for (long long off = 0; off < count; off += f->n_max) {
-    const int nb = (int)std::min<long long>(f->n_max, count - off);
+  for (long long off = 0; off < count; off += f->piece) {
+    const int nb = (int)std::min<long long>(f->piece, count - off);
     PV_KLAUNCH(&c->kprof, st, "k_fconfigs", 0.0, 0.0,
                k_fconfigs<<<(nb + 127) / 128, 128, 0, st>>>(nb, c->P.L1, c->P.L2, dS + off * N,
                                                            f->d_S32, f->d_csign, f->d_bad));
@@ -2534,14 +2535,27 @@ int peps_famp_create(int L1, int L2, int D, int chi, int n_max, int precision, v
     f->c = nullptr;
     return rc;
   };
-  int rc;
+  int rc, dev = 0, sms = 152;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  // A local energy takes about 120 amplitudes per configuration (6x6), all independent, so the engine
+  // holds eight configurations per SM however few chains a call has: 128 chains leave most of the
+  // chip idle.  The larger work buffers stay below 4 GiB and an eighth of the free memory.
+  f->piece = n_max;
+  {
+    size_t fr = 0, tot = 0;
+    cudaMemGetInfo(&fr, &tot);
+    const size_t per = batched_chain_bytes(&c->P), cap = std::min<size_t>(fr / 8, (size_t)4 << 30);
+    f->piece = (int)std::max<long long>(n_max, std::min<long long>(8LL * sms, (long long)(cap / per)));
+  }
+  c->P.n_chains = f->piece;   // of the engine's buffers
   if ((rc = dalloc(c, &f->d_toff16, (N + 1) * sizeof(long long)))) return bail(rc);
   if ((rc = dalloc(c, &f->d_toff32, (N + 1) * sizeof(long long)))) return bail(rc);
   if ((rc = dalloc(c, &f->d_th16, (size_t)f->n16 * sizeof(double)))) return bail(rc);
   if ((rc = dalloc(c, (unsigned char**)&f->d_th32, (size_t)f->toff32[N] * real))) return bail(rc);
   if ((rc = dalloc(c, &f->d_S16, (size_t)n_max * N))) return bail(rc);
-  if ((rc = dalloc(c, &f->d_S32, (size_t)n_max * N))) return bail(rc);
-  if ((rc = dalloc(c, &f->d_csign, (size_t)n_max))) return bail(rc);
+  if ((rc = dalloc(c, &f->d_S32, (size_t)f->piece * N))) return bail(rc);
+  if ((rc = dalloc(c, &f->d_csign, (size_t)f->piece))) return bail(rc);
   if ((rc = dalloc(c, &f->d_sg, (size_t)n_max))) return bail(rc);
   if ((rc = dalloc(c, &f->d_la, (size_t)n_max * sizeof(double)))) return bail(rc);
   if ((rc = dalloc(c, &f->d_bad, sizeof(int)))) return bail(rc);
@@ -2549,9 +2563,6 @@ int peps_famp_create(int L1, int L2, int D, int chi, int n_max, int precision, v
   if (cudaMemcpy(f->d_toff16, f->toff16.data(), (N + 1) * sizeof(long long), cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(f->d_toff32, f->toff32.data(), (N + 1) * sizeof(long long), cudaMemcpyHostToDevice) != cudaSuccess)
     return bail(PEPS_ECUDA);
-  int dev = 0, sms = 152;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (precision == PEPS_FP64) {
     f->b64 = new BatchImpl<double>();
     c->batch.reset(f->b64);
