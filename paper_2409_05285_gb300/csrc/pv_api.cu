@@ -951,7 +951,7 @@ int init_runner_t(peps_ctx* c, int sms, BatchImpl<T>* b, int Dn, const T* theta,
       e = cudaFuncSetAttribute(kb_trunc_wide<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, tw_max);
       b->be.trunc_wide_max = e == cudaSuccess ? tw_max : 0;
       if (e != cudaSuccess) cudaGetLastError();
-      e = cudaFuncSetAttribute(kb_chol<T, 1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, tw_max);
+      e = cudaFuncSetAttribute(kb_chol<T, 512>, cudaFuncAttributeMaxDynamicSharedMemorySize, tw_max);
       b->be.chol_wide_max = e == cudaSuccess ? tw_max : 0;
       if (e != cudaSuccess) cudaGetLastError();
     }
