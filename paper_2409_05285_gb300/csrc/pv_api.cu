@@ -968,12 +968,7 @@ int init_runner_t(peps_ctx* c, int sms, BatchImpl<T>* b, int Dn, const T* theta,
     // also takes the right factors from the Gram matrix
     if ((rc = dalloc(c, &b->be.tc_err, sizeof(int)))) return rc;
     cudaError_t e = cudaMemsetAsync(b->be.tc_err, 0, sizeof(int), c->stream);
-    auto big = [&](auto k) {
-      if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    };
-    big(kb_gemm_tc<8, 4, 4>);
-    big(kb_gemm_tc<4, 4, 5>);
-    big(kb_gemm_tc<4, 8, 4>);
+    if (e == cudaSuccess) e = tc_setup();
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(kb_chol<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     if (e != cudaSuccess) return fail(c, PEPS_ECUDA, std::string("tensor-core setup: ") + cudaGetErrorString(e));

@@ -2041,9 +2041,7 @@ struct CudaBE {
                        kern<<<gr, TC_THREADS, bytes, st>>>(t, out, os, swap ? B : A, swap ? A : B, n, tilesN, tc_err,
                                                            act));
           };
-          if (t.Kc == 32) go(kb_gemm_tc<8, 4, 4>, 4);
-          else if (t.TN <= 128) go(kb_gemm_tc<4, 4, 5>, 5);
-          else go(kb_gemm_tc<4, 8, 4>, 4);
+          tc_kernel(t, go);
           return;
         }
       }

@@ -49,12 +49,12 @@ inline void tc_shape(TcSpec& t, int kc_max) {
 // the quads of contraction indices (Kc / 4).  Every lane's vector is four contraction indices of
 // a row or, in a 4 x 4 block of an operand that is contiguous in its rows (TC_VEC_T), four rows
 // at four indices: transposed by naming, when it is stored.
-template <int NU>
-__device__ __forceinline__ void tc_load(float4 (&r)[NU], const float* __restrict__ src, int mode, bool kfast,
+template <int mode, int NU>
+__device__ __forceinline__ void tc_load(float4 (&r)[NU], const float* __restrict__ src, bool kfast,
                                          int rows, int lq, int k0, int K, const int* roff, const int* koff,
                                          int tid) {
   const int qn = 1 << lq;
-  if (mode == TC_VEC_K) {
+  if constexpr (mode == TC_VEC_K) {
 #pragma unroll
     for (int u = 0; u < NU; ++u) {
       const int e = tid + u * TC_THREADS;
@@ -65,7 +65,7 @@ __device__ __forceinline__ void tc_load(float4 (&r)[NU], const float* __restrict
         if (ro >= 0) r[u] = __ldg((const float4*)(src + ro + koff[k]));
       }
     }
-  } else if (mode == TC_VEC_T) {
+  } else if constexpr (mode == TC_VEC_T) {
 #pragma unroll
     for (int b = 0; b < NU / 4; ++b) {
       const int e = tid + b * TC_THREADS;
@@ -98,9 +98,9 @@ __device__ __forceinline__ void tc_load(float4 (&r)[NU], const float* __restrict
 
 // Rounds the registers of tc_load to TF32 and stores them in the K-major layout without swizzle
 // (and the rounding of the remainders to `lo` where it is given).
-template <int NU>
-__device__ __forceinline__ void tc_store(const float4 (&r)[NU], float* hi, float* lo, int mode, bool kfast, int rows,
-                                          int lq, int tid) {
+template <int mode, int NU>
+__device__ __forceinline__ void tc_store(const float4 (&r)[NU], float* hi, float* lo, bool kfast, int rows, int lq,
+                                         int tid) {
   const int qn = 1 << lq, gs = (qn << 5) + 4;
   auto put = [&](int rr, int q, float4 v) {
     const int e = (rr >> 3) * gs + (q << 5) + ((rr & 7) << 2);
@@ -108,7 +108,7 @@ __device__ __forceinline__ void tc_store(const float4 (&r)[NU], float* hi, float
     *(float4*)(hi + e) = h;
     if (lo) *(float4*)(lo + e) = tc_round4(make_float4(v.x - h.x, v.y - h.y, v.z - h.z, v.w - h.w));
   };
-  if (mode == TC_VEC_T) {
+  if constexpr (mode == TC_VEC_T) {
 #pragma unroll
     for (int b = 0; b < NU / 4; ++b) {
       const int e = tid + b * TC_THREADS;
@@ -131,7 +131,9 @@ __device__ __forceinline__ void tc_store(const float4 (&r)[NU], float* hi, float
   }
 }
 
-template <int NA, int NB, int MINB>
+// MP, MQ: the operands' gather forms (compiled apart: an item is some 350 instructions, and the
+// instruction cache pays for every path that lies between them).
+template <int NA, int NB, int MINB, int MP, int MQ>
 __global__ void __launch_bounds__(TC_THREADS, MINB) kb_gemm_tc(TcSpec t, float* C, long long cs, Operand<float> P,
                                                                Operand<float> Q, int n, int tilesN, int* err,
                                                                ChainList cl) {
@@ -193,8 +195,8 @@ __global__ void __launch_bounds__(TC_THREADS, MINB) kb_gemm_tc(TcSpec t, float* 
   uint32_t ph = 0u;
   float4 ra[NA], rb[NB];
   auto load = [&](const float* p, const float* q, int k0) {
-    tc_load(ra, p, t.modeP, kfP, rowsA, lq, k0, t.K, rowP, kPo, tid);
-    if (!t.sym) tc_load(rb, q, t.modeQ, kfQ, rowsB, lq, k0, t.K, colQ, kQo, tid);
+    tc_load<MP>(ra, p, kfP, rowsA, lq, k0, t.K, rowP, kPo, tid);
+    if (!t.sym) tc_load<MQ>(rb, q, kfQ, rowsB, lq, k0, t.K, colQ, kQo, tid);
   };
   auto desc = [&](uint32_t base, int kb) { return tc_desc(base + kb * 256, 128, (uint32_t)gs * 4u); };
   const float *pn = nullptr, *qn = nullptr;   // operands of the next chain: their addresses are formed
@@ -218,8 +220,8 @@ __global__ void __launch_bounds__(TC_THREADS, MINB) kb_gemm_tc(TcSpec t, float* 
   for (int k = blockIdx.y; k < n && !stop; k += gy) {
     bool good = true;
     for (int k0 = 0; k0 < t.K; k0 += Kc) {
-      tc_store(ra, As, Al, t.modeP, kfP, rowsA, lq, tid);
-      if (!t.sym) tc_store(rb, Bs, Bl, t.modeQ, kfQ, rowsB, lq, tid);
+      tc_store<MP>(ra, As, Al, kfP, rowsA, lq, tid);
+      if (!t.sym) tc_store<MQ>(rb, Bs, Bl, kfQ, rowsB, lq, tid);
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       tc_fence_before();
       __syncthreads();
@@ -274,6 +276,40 @@ __global__ void __launch_bounds__(TC_THREADS, MINB) kb_gemm_tc(TcSpec t, float* 
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(ncols) : "memory");
   }
   if (tid == 0 && abort_flag) atomicOr(err, stuck ? 3 : 1);
+}
+
+// f(kernel, resident CTAs per SM that its registers allow) for the variant of a spec.
+template <int NA, int NB, int MINB, typename F>
+void tc_modes(int mp, int mq, F&& f) {
+  auto q = [&](auto MP) {
+    if (mq == TC_VEC_K) f(kb_gemm_tc<NA, NB, MINB, MP.value, TC_VEC_K>, MINB);
+    else if (mq == TC_VEC_T) f(kb_gemm_tc<NA, NB, MINB, MP.value, TC_VEC_T>, MINB);
+    else f(kb_gemm_tc<NA, NB, MINB, MP.value, TC_SCALAR>, MINB);
+  };
+  if (mp == TC_VEC_K) q(std::integral_constant<int, TC_VEC_K>());
+  else if (mp == TC_VEC_T) q(std::integral_constant<int, TC_VEC_T>());
+  else q(std::integral_constant<int, TC_SCALAR>());
+}
+template <typename F>
+void tc_kernel(const TcSpec& t, F&& f) {
+  if (t.Kc == 32) tc_modes<8, 4, 4>(t.modeP, t.modeQ, f);
+  else if (t.TN <= 128) tc_modes<4, 4, 5>(t.modeP, t.modeQ, f);
+  else tc_modes<4, 8, 4>(t.modeP, t.modeQ, f);
+}
+// Shared memory of every variant.
+inline cudaError_t tc_setup() {
+  cudaError_t e = cudaSuccess;
+  TcSpec t;
+  for (int v = 0; v < 27; ++v) {
+    t.Kc = v < 9 ? 32 : 16;
+    t.TN = v < 18 ? 128 : 256;
+    t.modeP = v / 3 % 3;
+    t.modeQ = v % 3;
+    tc_kernel(t, [&](auto k, int) {
+      if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    });
+  }
+  return e;
 }
 
 #endif  // __CUDACC__
