@@ -1179,10 +1179,13 @@ inline void bond_lists(int L1, int L2, double J1, double J2, std::vector<int>& b
 }  // namespace pv
 
 #include "pv_tc.cuh"
-#include "pv_gemm.cuh"
 
 #if defined(__CUDACC__)
 #include "pv_prof.cuh"
+#endif
+#include "pv_gemm.cuh"
+
+#if defined(__CUDACC__)
 #include "pv_jacobi.cuh"
 #include "pv_prog.cuh"
 namespace pv {
@@ -1193,6 +1196,8 @@ constexpr int LQ_THREADS = 512;   // threads of the shared-memory Householder ke
 template <typename T>
 __global__ void __launch_bounds__(256) kb_ein(MSpec m, T* out, long long os, Operand<T> A,
                                               Operand<T> B, int n, int quad, ChainList cl) {
+  pdl_go();
+  pdl_wait();
   if ((int)blockIdx.y >= cl.count(n)) return;
   const int s = cl.chain(blockIdx.y);
   const T* pa = A.at(s);
@@ -1245,6 +1250,8 @@ __global__ void __launch_bounds__(256) kb_gemm(GSpec g, T* C, long long cs, Oper
   const int per = (TM >> 2) * tnx;          // compute threads per sample
   const int slot = tid / per, loc = tid - slot * per;
   const int tx = loc % tnx, ty = loc / tnx;
+  pdl_go();
+  pdl_wait();
   n = cl.count(n);
   for (int sbase = blockIdx.y * G; sbase < n; sbase += gridDim.y * G) {
     const int ns = min(G, n - sbase);
@@ -1684,6 +1691,8 @@ template <typename T>
 __global__ void __launch_bounds__(128, 6) kb_chol64(OpChol<T> op, int n) {
   __shared__ T lc[128];
   __shared__ T red[32];
+  pdl_go();
+  pdl_wait();
   for (int s = blockIdx.x; s < n; s += gridDim.x) chol64<T, 8>(op, s, lc, red);
 }
 
@@ -1747,6 +1756,8 @@ __global__ void __launch_bounds__(1024) kb_trunc_wide(OpTrunc<T> op, int n) {
 template <typename T>
 __global__ void __launch_bounds__(BT) kb_norm(OpNorm<T> op, int n) {
   __shared__ T red[32];
+  pdl_go();
+  pdl_wait();
   for (int s = blockIdx.x; s < n; s += gridDim.x) {
     op(s, red);
     __syncthreads();
@@ -1758,6 +1769,8 @@ template <typename T>
 __global__ void __launch_bounds__(256) kb_dot(OpDot<T> op, int n, ChainList cl) {
   const int k0 = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
+  pdl_go();
+  pdl_wait();
   if (k0 >= cl.count(n)) return;
   const int s = cl.chain(k0);
   const T* a = op.a + (long long)s * op.as;
@@ -1776,6 +1789,8 @@ constexpr int DOT_TILE = 2048;
 template <typename T>
 __global__ void __launch_bounds__(256) kb_dot_block(OpDot<T> op, int n, ChainList cl) {
   __shared__ T sa[DOT_TILE], sb[DOT_TILE];
+  pdl_go();
+  pdl_wait();
   if ((int)blockIdx.x >= cl.count(n)) return;
   const int s = cl.chain(blockIdx.x), tid = threadIdx.x;
   const T* a = op.a + (long long)s * op.as;
@@ -1813,6 +1828,8 @@ __global__ void __launch_bounds__(256) kb_dot_block(OpDot<T> op, int n, ChainLis
 
 template <typename F>
 __global__ void kb_elem(F f, int n) {
+  pdl_go();
+  pdl_wait();
   int s = blockIdx.x * blockDim.x + threadIdx.x;
   if (s < n) f(s);
 }
@@ -1822,6 +1839,8 @@ __global__ void kb_elem(F f, int n) {
 // kernels that read its last value have ended.
 static __global__ void __launch_bounds__(128) kb_sel_list(ElemSel f, int n, int* idx, int* cnt, int* zero) {
   const int s = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
+  pdl_go();
+  pdl_wait();
   bool v = false;
   if (s < n) {
     f(s);
@@ -1861,6 +1880,8 @@ static __global__ void kb_copyd(double* x, long long xs, int dst, int src, int n
 template <typename T>
 __global__ void kb_copy(T* dst, long long ds, const T* src, long long ss, long long len,
                         const int8_t* mask, int n) {
+  pdl_go();
+  pdl_wait();
   int s = blockIdx.y;
   if (s >= n || (mask && !mask[s])) return;
   long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -1999,6 +2020,11 @@ struct CudaBE {
            int n, bool exact = false) {
     GSpec gs = gemm_spec(raw);
     const int nw = act_n < 0 ? n : act_n;   // chains the profile counts
+    // An early start gains a few microseconds a launch (measured with it / without: 8x8 D=4, about 35
+    // and 70 MB a launch: sweep of 1024 chains 74 / 79 ms, evaluation of 2048 99 / 108; 6x6 Hubbard
+    // step 93 / 99), but the successor's waiting blocks cost a launch of 100 us more than that (10x10
+    // D=6 with every contraction early 980 ms, with none 945), so it ends at 96 MB.
+    const bool early = ein_bytes(raw, A, B, n) <= 96e6;
     if (rec) {
       rec->bytes += ein_bytes(raw, A, B, 1);
       if constexpr (std::is_same<T, float>::value) {
@@ -2038,7 +2064,7 @@ struct CudaBE {
             gy = gy > 65535 ? 65535 : gy;
             dim3 gr(tilesM * tilesN, (unsigned)gy);
             PV_KLAUNCH(prof, st, "kb_gemm_tc", ein_bytes(raw, A, B, nw), 2.0 * raw.total * raw.kprod * nw,
-                       kern<<<gr, TC_THREADS, bytes, st>>>(t, out, os, swap ? B : A, swap ? A : B, n, tilesN, tc_err,
+                       pdl_if(early, kern, gr, TC_THREADS, bytes, st, t, out, os, swap ? B : A, swap ? A : B, n, tilesN, tc_err,
                                                            act));
           };
           tc_kernel(t, go);
@@ -2072,14 +2098,14 @@ struct CudaBE {
       if (gy > 65535) gy = 65535;
       dim3 gr(tilesN * tilesM, gy);
       PV_KLAUNCH(prof, st, "kb_gemm", ein_bytes(raw, A, B, nw), 2.0 * raw.total * raw.kprod * nw,
-                 kb_gemm<T><<<gr, 256, bytes, st>>>(gs, out, os, A, B, n, TM, TN, KC, tilesN, G, act));
+                 pdl_if(early, kb_gemm<T>, gr, 256, bytes, st, gs, out, os, A, B, n, TM, TN, KC, tilesN, G, act));
       return;
     }
     int quad = quad_ok(m) ? 1 : 0;
     long long work = quad ? (m.total >> 2) : m.total;
     dim3 g(gx(work, 256), n);
     PV_KLAUNCH(prof, st, "kb_ein", ein_bytes(raw, A, B, nw), 2.0 * raw.total * raw.kprod * nw,
-               kb_ein<T><<<g, 256, 0, st>>>(m, out, os, A, B, n, quad, act));
+               pdl(kb_ein<T>, g, 256, 0, st, m, out, os, A, B, n, quad, act));
   }
   void lq(OpLq<T> op, int n) {
     const int K = op.m < op.nn ? op.m : op.nn;
@@ -2193,7 +2219,7 @@ struct CudaBE {
     if (op.m <= 64) {
       const int grid = n < 6 * sms ? n : 6 * sms;   // resident at once
       PV_KLAUNCH(prof, st, "kb_chol", (double)n * 2.0 * op.m * op.m * sizeof(T),
-                 (double)op.m * op.m * op.m / 3.0 * n, (kb_chol64<T><<<grid, 128, 0, st>>>(op, n)));
+                 (double)op.m * op.m * op.m / 3.0 * n, (pdl(kb_chol64<T>, grid, 128, 0, st, op, n)));
       return;
     }
     if (bytes > 96 * 1024 && (int)bytes <= chol_wide_max) {
@@ -2218,7 +2244,7 @@ struct CudaBE {
       o.g.i[0] = op.lstride;
       return;
     }
-    PV_KLAUNCH(prof, st, "kb_norm", 0.0, 0.0, kb_norm<T><<<gblocks(n), BT, 0, st>>>(op, n));
+    PV_KLAUNCH(prof, st, "kb_norm", 0.0, 0.0, pdl(kb_norm<T>, gblocks(n), BT, 0, st, op, n));
   }
   void dot(OpDot<T> op, int n) {
     if (rec) {
@@ -2232,10 +2258,10 @@ struct CudaBE {
       return;
     }
     if (op.len >= DOT_TILE && n <= 16 * sms) {
-      PV_KLAUNCH(prof, st, "kb_dot", 0.0, 0.0, kb_dot_block<T><<<n, 256, 0, st>>>(op, n, act));
+      PV_KLAUNCH(prof, st, "kb_dot", 0.0, 0.0, pdl(kb_dot_block<T>, n, 256, 0, st, op, n, act));
       return;
     }
-    PV_KLAUNCH(prof, st, "kb_dot", 0.0, 0.0, kb_dot<T><<<gx(n, 8), 256, 0, st>>>(op, n, act));
+    PV_KLAUNCH(prof, st, "kb_dot", 0.0, 0.0, pdl(kb_dot<T>, gx(n, 8), 256, 0, st, op, n, act));
   }
   void set(T* x, long long xs, long long off, T v, int n) {
     if (rec) {
@@ -2289,7 +2315,7 @@ struct CudaBE {
       return;
     }
     dim3 g(gx(len, 256), n);
-    PV_KLAUNCH(prof, st, "kb_copy", 0.0, 0.0, kb_copy<T><<<g, 256, 0, st>>>(dst, ds, src, ss, len, mask, n));
+    PV_KLAUNCH(prof, st, "kb_copy", 0.0, 0.0, pdl(kb_copy<T>, g, 256, 0, st, dst, ds, src, ss, len, mask, n));
   }
   void diag(const uint8_t* S, int n, double* es, double* ea) {
     if (rec) {
@@ -2300,7 +2326,7 @@ struct CudaBE {
       o.g.i[0] = nb;
       return;
     }
-    PV_KLAUNCH(prof, st, "kb_elem_diag", 0.0, 0.0, kb_elem<<<gx(n, 128), 128, 0, st>>>(ElemDiag{S, N, nb, bi, bj, bJ, es, ea}, n));
+    PV_KLAUNCH(prof, st, "kb_elem_diag", 0.0, 0.0, pdl(kb_elem<ElemDiag>, gx(n, 128), 128, 0, st, ElemDiag{S, N, nb, bi, bj, bJ, es, ea}, n));
   }
   void amp(const T* val, long long vs, const double* lsd, int lstride, double* la, int8_t* sg, int n) {
     if (rec) {
@@ -2311,7 +2337,7 @@ struct CudaBE {
       o.g.i[0] = lstride;
       return;
     }
-    PV_KLAUNCH(prof, st, "kb_elem_amp", 0.0, 0.0, kb_elem<<<gx(n, 128), 128, 0, st>>>(ElemAmp<T>{val, vs, lsd, lstride, la, sg}, n));
+    PV_KLAUNCH(prof, st, "kb_elem_amp", 0.0, 0.0, pdl(kb_elem<ElemAmp<T>>, gx(n, 128), 128, 0, st, ElemAmp<T>{val, vs, lsd, lstride, la, sg}, n));
   }
   void writeO(OT* O, long long No, long long o_off, const T* env, long long es, long long sz,
               const T* val, long long vs, int n) {
@@ -2338,11 +2364,11 @@ struct CudaBE {
       return;
     }
     if (f.kind == 0) {   // a flip changes every chain
-      PV_KLAUNCH(prof, st, "kb_elem_sel", 0.0, 0.0, kb_elem<<<gx(n, 128), 128, 0, st>>>(f, n));
+      PV_KLAUNCH(prof, st, "kb_elem_sel", 0.0, 0.0, pdl(kb_elem<ElemSel>, gx(n, 128), 128, 0, st, f, n));
       return;
     }
     PV_KLAUNCH(prof, st, "kb_elem_sel", 0.0, 0.0,
-               kb_sel_list<<<gx(n, 128), 128, 0, st>>>(f, n, act_idx, act_cnt + act_cur, act_cnt + (act_cur ^ 1)));
+               pdl(kb_sel_list, gx(n, 128), 128, 0, st, f, n, act_idx, act_cnt + act_cur, act_cnt + (act_cur ^ 1)));
     act_cur ^= 1;
   }
   void ratio(const T* num, const T* den, long long dens, const int8_t* valid, double coef,
@@ -2356,7 +2382,7 @@ struct CudaBE {
       o.g.d = coef;
       return;
     }
-    PV_KLAUNCH(prof, st, "kb_elem_ratio", 0.0, 0.0, kb_elem<<<gx(n, 128), 128, 0, st>>>(ElemRatio<T>{num, den, dens, valid, coef, e}, n));
+    PV_KLAUNCH(prof, st, "kb_elem_ratio", 0.0, 0.0, pdl(kb_elem<ElemRatio<T>>, gx(n, 128), 128, 0, st, ElemRatio<T>{num, den, dens, valid, coef, e}, n));
   }
   void accept(ElemAccept<T> f, int n) {
     if (rec) {
@@ -2368,7 +2394,7 @@ struct CudaBE {
       o.g.i[2] = (int)f.id;
       return;
     }
-    PV_KLAUNCH(prof, st, "kb_elem_accept", 0.0, 0.0, kb_elem<<<gx(n, 128), 128, 0, st>>>(f, n));
+    PV_KLAUNCH(prof, st, "kb_elem_accept", 0.0, 0.0, pdl(kb_elem<ElemAccept<T>>, gx(n, 128), 128, 0, st, f, n));
   }
   // direct sampling (pv_direct.cuh): configuration fill, the candidate selector of every
   // chain, and one draw
@@ -2390,7 +2416,7 @@ struct CudaBE {
       rec->add(PG_DRAW).g.i[0] = f.i;
       return;
     }
-    PV_KLAUNCH(prof, st, "kb_elem_draw", 0.0, 0.0, kb_elem<<<gx(n, 128), 128, 0, st>>>(f, n));
+    PV_KLAUNCH(prof, st, "kb_elem_draw", 0.0, 0.0, pdl(kb_elem<ElemDraw<T>>, gx(n, 128), 128, 0, st, f, n));
   }
 };
 

@@ -62,7 +62,7 @@ __device__ __forceinline__ void tc_load(float4 (&r)[NU], const float* __restrict
       r[u] = make_float4(0.f, 0.f, 0.f, 0.f);
       if (rr < rows && k < K) {
         const int ro = roff[rr];
-        if (ro >= 0) r[u] = __ldg((const float4*)(src + ro + koff[k]));
+        if (ro >= 0) r[u] = *(const float4*)(src + ro + koff[k]);
       }
     }
   } else if constexpr (mode == TC_VEC_T) {
@@ -74,7 +74,7 @@ __device__ __forceinline__ void tc_load(float4 (&r)[NU], const float* __restrict
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         r[4 * b + i] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (ro >= 0 && kb + i < K) r[4 * b + i] = __ldg((const float4*)(src + ro + koff[kb + i]));
+        if (ro >= 0 && kb + i < K) r[4 * b + i] = *(const float4*)(src + ro + koff[kb + i]);
       }
     }
   } else {
@@ -89,7 +89,7 @@ __device__ __forceinline__ void tc_load(float4 (&r)[NU], const float* __restrict
       if (ro >= 0) {
 #pragma unroll
         for (int i = 0; i < 4; ++i)
-          if (kb + i < K) v[i] = __ldg(src + ro + koff[kb + i]);
+          if (kb + i < K) v[i] = src[ro + koff[kb + i]];
       }
       r[u] = make_float4(v[0], v[1], v[2], v[3]);
     }
@@ -187,6 +187,8 @@ __global__ void __launch_bounds__(TC_THREADS, MINB) kb_gemm_tc(TcSpec t, float* 
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  pdl_go();
+  pdl_wait();
   const uint32_t tmem = tslot, idesc = tc_idesc(TC_ROWS, TN);
   const uint32_t a = tc_smem_addr(As), b = tc_smem_addr(Bs);
   const uint32_t al = t.split ? tc_smem_addr(Al) : 0, bl = t.split ? tc_smem_addr(Bl) : 0;

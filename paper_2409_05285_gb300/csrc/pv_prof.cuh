@@ -4,6 +4,7 @@
 #ifndef PV_PROF_CUH
 #define PV_PROF_CUH
 #include <cuda_runtime.h>
+#include <utility>
 #include <cstring>
 #include <string>
 #include <vector>
@@ -83,6 +84,38 @@ struct KProf {
     acc.clear();
   }
 };
+
+// Programmatic dependent launch: the batched engine is thousands of short kernels in a row, and a
+// kernel's launch, its index tables and its tensor-memory allocation need nothing of the one before.
+// A kernel launched with pdl() may start while its predecessor in the stream ends, and calls pdl_wait()
+// before its first access to device memory (the wait covers the predecessor's completion and its writes,
+// and, as the predecessor waited itself, everything before).  pdl_go() lets the successor start;
+// a kernel that allocates tensor memory calls it only when it holds its columns (a successor's
+// block that took them first would wait for this kernel's end).  Launched without pdl() both do
+// nothing.
+#if defined(__CUDACC__)
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_go() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <typename... P, typename... A>
+inline void pdl_if(bool early, void (*kern)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, A&&... a) {
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c = {};
+  c.gridDim = grid;
+  c.blockDim = dim3(threads);
+  c.dynamicSmemBytes = smem;
+  c.stream = st;
+  c.attrs = at;
+  c.numAttrs = early ? 1 : 0;
+  cudaLaunchKernelEx(&c, kern, P(a)...);
+}
+template <typename... P, typename... A>
+inline void pdl(void (*kern)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, A&&... a) {
+  pdl_if(true, kern, grid, threads, smem, st, std::forward<A>(a)...);
+}
+#endif
 
 // Brackets one launch statement: counts it and, when profiling, times it.
 #define PV_KLAUNCH(prof, st, name, bytes, flops, ...) \
