@@ -1923,7 +1923,12 @@ inline bool op_same(const Operand<T>& a, const Operand<T>& b) {
          a.N == b.N && a.sel == b.sel;
 }
 
-// Whether every chain's slice of a float operand starts on a 16-byte boundary.
+// Whether every chain's slice of a float operand starts on an 8-byte (16-byte) boundary.
+inline bool op_al8(const Operand<float>& o) {
+  if ((uintptr_t)o.base % 8) return false;
+  if (o.mode == OP_BATCH) return o.stride % 2 == 0;
+  return o.site_off % 2 == 0 && o.site_sz % 2 == 0;
+}
 inline bool op_al16(const Operand<float>& o) {
   if ((uintptr_t)o.base % 16) return false;
   if (o.mode == OP_BATCH) return o.stride % 4 == 0;
@@ -2046,8 +2051,8 @@ struct CudaBE {
       TcSpec t;
       bool swap = false;
       if (tc && tc_plan(gs, t, swap, tc_min_rows)) {
-        tc_forms(t, op_al16(swap ? B : A), op_al16(swap ? A : B),
-                 ((uintptr_t)out % 16 == 0) && os % 4 == 0);
+        tc_forms(t, op_al16(swap ? B : A), op_al16(swap ? A : B), ((uintptr_t)out % 16 == 0) && os % 4 == 0,
+                 op_al8(swap ? B : A), op_al8(swap ? A : B));
         t.split = (exact || tc_split) ? 1 : 0;   // float32-accurate products (3xTF32)
         if (tc_form_override) tc_form_override(t);
         t.sym = tc_symmetric(t, op_same(A, B)) ? 1 : 0;

@@ -50,7 +50,7 @@ inline void tc_shape(TcSpec& t, int kc_max) {
 // a row or, in a 4 x 4 block of an operand that is contiguous in its rows (TC_VEC_T), four rows
 // at four indices: transposed by naming, when it is stored.
 template <int mode, int NU>
-__device__ __forceinline__ void tc_load(float4 (&r)[NU], const float* __restrict__ src, bool kfast,
+__device__ __forceinline__ void tc_load(float4 (&r)[NU], const float* __restrict__ src, bool kfast, bool pair,
                                          int rows, int lq, int k0, int K, const int* roff, const int* koff,
                                          int tid) {
   const int qn = 1 << lq;
@@ -87,9 +87,19 @@ __device__ __forceinline__ void tc_load(float4 (&r)[NU], const float* __restrict
       const int ro = rr < rows ? roff[rr] : -1;
       float v[4] = {0.f, 0.f, 0.f, 0.f};
       if (ro >= 0) {
+        if (pair) {
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
-          if (kb + i < K) v[i] = src[ro + koff[kb + i]];
+          for (int i = 0; i < 4; i += 2)
+            if (kb + i < K) {
+              const float2 w = *(const float2*)(src + ro + koff[kb + i]);
+              v[i] = w.x;
+              v[i + 1] = w.y;
+            }
+        } else {
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+            if (kb + i < K) v[i] = src[ro + koff[kb + i]];
+        }
       }
       r[u] = make_float4(v[0], v[1], v[2], v[3]);
     }
@@ -197,8 +207,8 @@ __global__ void __launch_bounds__(TC_THREADS, MINB) kb_gemm_tc(TcSpec t, float* 
   uint32_t ph = 0u;
   float4 ra[NA], rb[NB];
   auto load = [&](const float* p, const float* q, int k0) {
-    tc_load<MP>(ra, p, kfP, rowsA, lq, k0, t.K, rowP, kPo, tid);
-    if (!t.sym) tc_load<MQ>(rb, q, kfQ, rowsB, lq, k0, t.K, colQ, kQo, tid);
+    tc_load<MP>(ra, p, kfP, t.pairP, rowsA, lq, k0, t.K, rowP, kPo, tid);
+    if (!t.sym) tc_load<MQ>(rb, q, kfQ, t.pairQ, rowsB, lq, k0, t.K, colQ, kQo, tid);
   };
   auto desc = [&](uint32_t base, int kb) { return tc_desc(base + kb * 256, 128, (uint32_t)gs * 4u); };
   const float *pn = nullptr, *qn = nullptr;   // operands of the next chain: their addresses are formed

@@ -25,6 +25,7 @@ struct TcSpec {
   int TN;                    // tile width: a multiple of 16, at most 256
   int Kc;                    // contraction chunk: 8, 16 or 32 (tc_shape)
   int modeP, modeQ;          // operand gather forms (TC_SCALAR, TC_VEC_K, TC_VEC_T)
+  int pairP, pairQ;          // TC_SCALAR: pairs of contraction indices are adjacent and 8-byte aligned
   int vecC;                  // 16-byte stores of four consecutive columns of C
   int split;                 // 3xTF32: operands as hi + lo TF32 parts, products hi.hi + hi.lo + lo.hi
   int sym;                   // Q is P with the same index maps (C = P P^T, one tile): the B
@@ -65,7 +66,7 @@ inline bool tc_plan(const GSpec& g, TcSpec& t, bool& swap, int tc_min_rows = 64)
   t.TN = n16 < 256 ? n16 : 256;
   t.Kc = 8;
   t.modeP = t.modeQ = TC_SCALAR;
-  t.vecC = 0;
+  t.vecC = t.pairP = t.pairQ = 0;
   t.split = 0;
   t.sym = 0;
   t.no_mma = 0;
@@ -93,23 +94,47 @@ inline bool tc_all4(const int* st, int n) {
 // Operand form: 16-byte loads along the contraction index or along the rows when the
 // operand is unit-stride there in blocks of four and every other stride keeps 16-byte
 // alignment (`al`: the operand's base and per-chain offsets are multiples of 16 bytes).
+// Length of the contiguous run of the trailing dims (0 unless the last is unit-stride); d: its first dim.
+inline int tc_run(int n, const int* sz, const int* st, int& d) {
+  d = n - 1;
+  if (n == 0 || st[n - 1] != 1) return 0;
+  int run = sz[d];
+  while (d > 0 && st[d - 1] == st[d] * sz[d]) run *= sz[--d];
+  return run;
+}
+
 inline int tc_mode(bool al, int nr, const int* rsz, const int* rst, int nk, const int* ksz,
                    const int* kst) {
   if (!al) return TC_SCALAR;
-  if (nk > 0 && kst[nk - 1] == 1 && ksz[nk - 1] % 4 == 0 && tc_all4(kst, nk - 1) &&
-      tc_all4(rst, nr))
-    return TC_VEC_K;
-  if (nr > 0 && rst[nr - 1] == 1 && rsz[nr - 1] % 4 == 0 && tc_all4(rst, nr - 1) &&
-      tc_all4(kst, nk))
-    return TC_VEC_T;
+  int d = 0, run = tc_run(nk, ksz, kst, d);
+  if (run && run % 4 == 0 && tc_all4(kst, d) && tc_all4(rst, nr)) return TC_VEC_K;
+  run = tc_run(nr, rsz, rst, d);
+  if (run && run % 4 == 0 && tc_all4(rst, d) && tc_all4(kst, nk)) return TC_VEC_T;
   return TC_SCALAR;
 }
 
-inline void tc_forms(TcSpec& t, bool p_al, bool q_al, bool c_al) {
+// Whether an element-wise operand can be loaded two contraction indices at a time (`al8`: base and
+// per-chain offsets are multiples of 8 bytes): contiguous in runs of even length, as the bonds of
+// D = 6 are.
+inline int tc_pairs(bool al8, int nr, const int* rst, int nk, const int* ksz, const int* kst) {
+  if (!al8 || nk == 0 || kst[nk - 1] != 1 || ksz[nk - 1] % 2) return 0;
+  for (int d = 0; d < nr; ++d)
+    if (rst[d] % 2) return 0;
+  for (int d = 0; d < nk - 1; ++d)
+    if (kst[d] % 2) return 0;
+  return 1;
+}
+
+inline void tc_forms(TcSpec& t, bool p_al, bool q_al, bool c_al, bool p_al8 = false, bool q_al8 = false) {
   t.modeP = tc_mode(p_al, t.nr, t.rs, t.rP, t.nk, t.ks, t.kP);
   t.modeQ = tc_mode(q_al, t.nc, t.cs, t.cQ, t.nk, t.ks, t.kQ);
-  t.vecC = (c_al && t.nc > 0 && t.cC[t.nc - 1] == 1 && t.cs[t.nc - 1] % 4 == 0 &&
-            tc_all4(t.cC, t.nc - 1) && tc_all4(t.rC, t.nr)) ? 1 : 0;
+  t.pairP = t.modeP == TC_SCALAR && tc_pairs(p_al8, t.nr, t.rP, t.nk, t.ks, t.kP);
+  t.pairQ = t.modeQ == TC_SCALAR && tc_pairs(q_al8, t.nc, t.cQ, t.nk, t.ks, t.kQ);
+  // four consecutive columns are adjacent in C when the trailing column dims that are contiguous
+  // there together hold a multiple of four (6 x 6 bond pairs at D = 6)
+  int d = 0;
+  const int run = tc_run(t.nc, t.cs, t.cC, d);
+  t.vecC = c_al && run && run % 4 == 0 && tc_all4(t.cC, d) && tc_all4(t.rC, t.nr) ? 1 : 0;
 }
 
 PV_HD int tc_cols(int TN) {
