@@ -362,7 +362,8 @@ int peps_restore(peps_ctx* ctx, const char* path);
 double peps_time(const peps_ctx* ctx);
 
 /* Device counters of the last peps_eval_batch / peps_mc_sweep launch: algorithmic
- * flops (contractions, Householder, Jacobi), Jacobi sweeps. */
+ * flops (contractions, Householder, Jacobi; a proposal's contractions count for every chain, also
+ * where its exchange changes nothing and they are left out), Jacobi sweeps. */
 int peps_last_counters(peps_ctx* ctx, double* flops, int64_t* jacobi_sweeps);
 
 /* Kernel launches this context has made since peps_init (every kernel of the library). */
@@ -370,9 +371,9 @@ long long peps_launches(const peps_ctx* ctx);
 
 /* Autotuner of the batched engine's launch shapes, keyed on the problem geometry (d^2 = 4,
  * D, chi, L1, L2, precision).  peps_autotune times `reps` evaluations of (at most 8192 of)
- * the context's chains per candidate (coordinate descent over the tensor-core grid size,
- * the operand stage count, the contraction chunk, the tensor-core kernel form, the chains
- * per FFMA block; only the last one without tensor cores) and keeps the fastest; the choice is stored in a process-wide table that later
+ * the context's chains per candidate (coordinate descent over the tensor-core grid size, the
+ * contraction chunk, the chains per FFMA block and the truncation's threads; only the last two
+ * without tensor cores) and keeps the fastest; the choice is stored in a process-wide table that later
  * contexts of the same geometry start from.  No candidate changes any result.  reps = 0
  * only reports the current choice.  With at most 8192 chains the chain buffers hold an
  * evaluation of the current state on return; otherwise evaluate before peps_sr_step.  `out` (caller-owned, may be NULL)

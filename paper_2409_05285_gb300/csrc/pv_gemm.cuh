@@ -11,15 +11,17 @@
 //
 // What bounds it: the operands and results of most contractions are 4 to 64 KB a chain, so the
 // instructions that gather an element and the latency of a chain's round trip cost more than its
-// bytes (8x8 D=4 chi=16: 2.5 TB/s of the operands' and results' bytes) or its MMAs.  Hence
+// bytes (8x8 D=4 chi=16, 8192 chains: 2.5 to 3 TB/s of the operands' and results') or its MMAs.  Hence
 //  - every lane moves 16 bytes at a time, contiguous rows included (4 x 4 blocks transposed in
 //    registers; the former kernels copied those 4 bytes at a time), index arithmetic is shifts
 //    (chunks are powers of two) and offsets come from tables;
 //  - one stage and one accumulator: with chunks this small more CTAs on an SM (four to five)
 //    overlap a round trip better than a second stage in each.
-// Measured, 8x8 D=4 chi=16 step of 8192 chains 864 -> 668 ms, 10x10 D=6 chi=36 evaluation of 192
-// chains 1330 -> 1176, 6x6 direct draw of 8192 chains 91 -> 77 against the kernels this one replaced
-// (a register-staged one and a cp.async ring of 4- and 16-byte copies).
+// Measured against the kernels this one replaced (a register-staged one and a cp.async ring of 4-
+// and 16-byte copies): 8x8 D=4 chi=16 step of 8192 chains 864 -> 668 ms, 10x10 D=6 chi=36 evaluation
+// of 192 chains 1330 -> 1176, 6x6 direct draw of 8192 chains 91 -> 77.  The operand forms compiled
+// apart then took the 1555 contractions of an 8x8 evaluation of 2048 chains from 61 to 52 ms, and
+// merged contiguous dims with pairs the 10x10 evaluation from 940 to 845 ms.
 #ifndef PV_GEMM_CUH
 #define PV_GEMM_CUH
 #include <cstdint>

@@ -115,7 +115,7 @@ __device__ __forceinline__ void pg_fma_tiles(const PgFma& f, const T* A, const T
 // ------------------------------------------------------------------ tensor-core contraction
 
 // Operand chunk (rows row0 .. row0 + rows - 1 of `lim`, Kc = 4 << lq indices from k0 of K) into the
-// canonical K-major layout of tc_gather, rounded to TF32; the operand was written by this block,
+// canonical K-major layout without swizzle, rounded to TF32; the operand was written by this block,
 // so its loads are plain ones.  Index tables `roff` (rows) and `koff`.
 __device__ __forceinline__ void pg_gather(float* dst, float* dlo, const float* src, int mode, int rows, int row0,
                                           int lim, int lq, int k0, int K, const int* __restrict__ roff,
