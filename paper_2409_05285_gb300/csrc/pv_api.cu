@@ -287,6 +287,14 @@ int grid_for(long long n, int threads, int cap = 152 * 16) {
 
 namespace {
 
+// Host data to the device, in order with what follows on `st`.  (cudaMemcpy of pageable memory may
+// return before the data has arrived, and a non-blocking stream does not wait for the default one.)
+cudaError_t upload(cudaStream_t st, void* dst, const void* src, size_t bytes) {
+  if (!bytes) return cudaSuccess;
+  const cudaError_t e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, st);
+  return e == cudaSuccess ? cudaStreamSynchronize(st) : e;   // src may go out of scope
+}
+
 // Type-erased batched engine of a context (float64 or float32 arithmetic).
 struct BatchIface {
   virtual ~BatchIface() {}
@@ -408,17 +416,21 @@ struct BatchImpl : BatchIface {
       pr.arena = (bd.need + 127) & ~(size_t)127;
       pr.bytes = bd.bytes;
       const size_t ob = bd.ops.size() * sizeof(PgOp), tb = (bd.tab.size() + 4) * sizeof(int);
+      // another thread may be capturing a stream of its own: an allocation here is no part of that
+      cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+      cudaThreadExchangeStreamCaptureMode(&mode);
       cudaError_t e = cudaMalloc((void**)&pr.d_ops, ob);
       if (e == cudaSuccess) e = cudaMalloc((void**)&pr.d_tab, tb);
-      if (e == cudaSuccess) e = cudaMemcpy(pr.d_ops, bd.ops.data(), ob, cudaMemcpyHostToDevice);
-      if (e == cudaSuccess && !bd.tab.empty())
-        e = cudaMemcpy(pr.d_tab, bd.tab.data(), bd.tab.size() * sizeof(int), cudaMemcpyHostToDevice);
-      if (e != cudaSuccess) {   // no room: the batched launches need none
-        cudaGetLastError();
+      cudaThreadExchangeStreamCaptureMode(&mode);
+      if (e == cudaSuccess) e = upload(be.st, pr.d_ops, bd.ops.data(), ob);
+      if (e == cudaSuccess) e = upload(be.st, pr.d_tab, bd.tab.data(), bd.tab.size() * sizeof(int));
+      if (e != cudaSuccess) {
         if (pr.d_ops) cudaFree(pr.d_ops);
         if (pr.d_tab) cudaFree(pr.d_tab);
         pr = PgProgram();
         pr.bad = true;
+        if (e != cudaErrorMemoryAllocation) return nullptr;   // the caller reports the error
+        cudaGetLastError();   // no room: the batched launches need none
       }
       break;
     }
@@ -823,7 +835,7 @@ int batch_status(peps_ctx* c, BatchIface* eng = nullptr) {
   int h = 0;
   PV_CUDA(c, cudaMemcpy(&h, d, sizeof(int), cudaMemcpyDeviceToHost));
   if (!h) return PEPS_OK;
-  PV_CUDA(c, cudaMemset(d, 0, sizeof(int)));
+  PV_CUDA(c, cudaMemsetAsync(d, 0, sizeof(int), c->stream));
   if (h & 2)
     return fail(c, PEPS_ETIMEOUT,
                 "tensor-core contraction: completion wait and its grace wait ran out; an MMA may "
@@ -913,7 +925,7 @@ int init_runner_t(peps_ctx* c, int sms, BatchImpl<T>* b, int Dn, const T* theta,
   if ((rc = dalloc(c, &b->d_sweep, sizeof(uint32_t)))) return rc;
   if (!c->d_jflops) {
     if ((rc = dalloc(c, &c->d_jflops, sizeof(double)))) return rc;
-    PV_CUDA(c, cudaMemset(c->d_jflops, 0, sizeof(double)));
+    PV_CUDA(c, cudaMemsetAsync(c->d_jflops, 0, sizeof(double), c->stream));
   }
   b->jflops_dev = c->d_jflops;
   if ((rc = dalloc(c, &b->ea_tmp, (size_t)chunk * sizeof(double)))) return rc;
@@ -926,11 +938,9 @@ int init_runner_t(peps_ctx* c, int sms, BatchImpl<T>* b, int Dn, const T* theta,
   if ((rc = dalloc(c, &dbi, nb * sizeof(int)))) return rc;
   if ((rc = dalloc(c, &dbj, nb * sizeof(int)))) return rc;
   if ((rc = dalloc(c, &dbJ, nb * sizeof(double)))) return rc;
-  if (!bi.empty()) {
-    cudaMemcpy(dbi, bi.data(), bi.size() * sizeof(int), cudaMemcpyHostToDevice);
-    cudaMemcpy(dbj, bj.data(), bj.size() * sizeof(int), cudaMemcpyHostToDevice);
-    cudaMemcpy(dbJ, bJ.data(), bJ.size() * sizeof(double), cudaMemcpyHostToDevice);
-  }
+  PV_CUDA(c, upload(c->stream, dbi, bi.data(), bi.size() * sizeof(int)));
+  PV_CUDA(c, upload(c->stream, dbj, bj.data(), bj.size() * sizeof(int)));
+  PV_CUDA(c, upload(c->stream, dbJ, bJ.data(), bJ.size() * sizeof(double)));
   b->be.st = c->stream;
   b->be.prof = &c->kprof;
   b->be.bi = dbi;
@@ -1020,7 +1030,7 @@ int make_direct_t(peps_ctx* c, int sms) {
   }
   PV_TRY(dalloc(c, (T**)&c->d_theta2, (size_t)c->toff2[N] * sizeof(T)));
   PV_TRY(dalloc(c, &c->d_toff2, (size_t)(N + 1) * sizeof(long long)));
-  PV_CUDA(c, cudaMemcpy(c->d_toff2, c->toff2.data(), (N + 1) * sizeof(long long), cudaMemcpyHostToDevice));
+  PV_CUDA(c, upload(c->stream, c->d_toff2, c->toff2.data(), (N + 1) * sizeof(long long)));
   PV_TRY(dalloc(c, &c->d_logq, (size_t)P->n_chains * sizeof(double)));
   PV_TRY(dalloc(c, &c->d_u, (size_t)P->n_chains * N * sizeof(double)));
   auto* b = new BatchImpl<T>();
@@ -2019,7 +2029,7 @@ int peps_profile(peps_ctx* c, int enable) {
     c->kprof.reset();
     c->kprof.on = true;
     c->kprof.gemm_only = enable == 2;
-    if (c->d_jflops) PV_CUDA(c, cudaMemset(c->d_jflops, 0, sizeof(double)));
+    if (c->d_jflops) PV_CUDA(c, cudaMemsetAsync(c->d_jflops, 0, sizeof(double), c->stream));
   } else {
     c->kprof.fold();
     c->kprof.on = false;
@@ -2354,8 +2364,8 @@ int famp_energies(peps_famp* f, int nb, double t_hop, double U, double mu) {
     f->nbonds = (int)bi.size();
     PV_TRY(dalloc(c, &f->d_bi, bi.size() * sizeof(int)));
     PV_TRY(dalloc(c, &f->d_bj, bj.size() * sizeof(int)));
-    PV_CUDA(c, cudaMemcpy(f->d_bi, bi.data(), bi.size() * sizeof(int), cudaMemcpyHostToDevice));
-    PV_CUDA(c, cudaMemcpy(f->d_bj, bj.data(), bj.size() * sizeof(int), cudaMemcpyHostToDevice));
+    PV_CUDA(c, upload(c->stream, f->d_bi, bi.data(), bi.size() * sizeof(int)));
+    PV_CUDA(c, upload(c->stream, f->d_bj, bj.data(), bj.size() * sizeof(int)));
     PV_TRY(dalloc(c, &f->d_es, (size_t)f->n_max * sizeof(double)));
     PV_TRY(dalloc(c, &f->d_ea, (size_t)f->n_max * sizeof(double)));
     PV_TRY(dalloc(c, &f->d_cnt, (size_t)f->n_max * sizeof(int)));
@@ -2400,7 +2410,7 @@ int famp_orows_alloc(peps_famp* f) {
   const size_t real = f->b64 ? sizeof(double) : sizeof(float);
   PV_TRY(dalloc(c, (unsigned char**)&f->d_O, (size_t)f->n_max * c->No * real));
   PV_TRY(dalloc(c, &f->d_ooff, (N + 1) * sizeof(long long)));
-  PV_CUDA(c, cudaMemcpy(f->d_ooff, c->ooff.data(), (N + 1) * sizeof(long long), cudaMemcpyHostToDevice));
+  PV_CUDA(c, upload(c->stream, f->d_ooff, c->ooff.data(), (N + 1) * sizeof(long long)));
   return PEPS_OK;
 }
 
@@ -2469,7 +2479,7 @@ int famp_sr_buffers(peps_famp* f) {
   for (int i = 0; i < N; ++i)
     for (long long o = c->ooff[i]; o < c->ooff[i + 1]; ++o) o2s[(size_t)o] = i;
   PV_TRY(dalloc(c, &f->d_o2site, (size_t)No * sizeof(int)));
-  PV_CUDA(c, cudaMemcpy(f->d_o2site, o2s.data(), (size_t)No * sizeof(int), cudaMemcpyHostToDevice));
+  PV_CUDA(c, upload(c->stream, f->d_o2site, o2s.data(), (size_t)No * sizeof(int)));
   for (double** v : {&f->d_w, &f->d_E, &f->d_y}) PV_TRY(dalloc(c, v, n * sizeof(double)));
   PV_TRY(dalloc(c, &f->d_ypart, nyb * sizeof(double)));
   for (double** v : {&f->d_obar, &f->d_g, &f->d_x, &f->d_r, &f->d_p, &f->d_q})
@@ -2555,8 +2565,8 @@ int peps_famp_create(int L1, int L2, int D, int chi, int n_max, int precision, v
   if ((rc = dalloc(c, &f->d_la, (size_t)n_max * sizeof(double)))) return bail(rc);
   if ((rc = dalloc(c, &f->d_bad, sizeof(int)))) return bail(rc);
   if ((rc = dalloc(c, &c->d_jsw, sizeof(unsigned long long)))) return bail(rc);
-  if (cudaMemcpy(f->d_toff16, f->toff16.data(), (N + 1) * sizeof(long long), cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMemcpy(f->d_toff32, f->toff32.data(), (N + 1) * sizeof(long long), cudaMemcpyHostToDevice) != cudaSuccess)
+  if (upload(c->stream, f->d_toff16, f->toff16.data(), (N + 1) * sizeof(long long)) != cudaSuccess ||
+      upload(c->stream, f->d_toff32, f->toff32.data(), (N + 1) * sizeof(long long)) != cudaSuccess)
     return bail(PEPS_ECUDA);
   if (precision == PEPS_FP64) {
     f->b64 = new BatchImpl<double>();
@@ -2635,7 +2645,7 @@ int peps_famp_set_strips(peps_famp* f, int enable) {
     const size_t real = f->b64 ? sizeof(double) : sizeof(float);
     PV_TRY(dalloc(c, (unsigned char**)&f->d_th64, (size_t)f->toff64[N] * real));
     PV_TRY(dalloc(c, &f->d_toff64, (N + 1) * sizeof(long long)));
-    PV_CUDA(c, cudaMemcpy(f->d_toff64, f->toff64.data(), (N + 1) * sizeof(long long), cudaMemcpyHostToDevice));
+    PV_CUDA(c, upload(c->stream, f->d_toff64, f->toff64.data(), (N + 1) * sizeof(long long)));
   }
   f->strips = enable != 0;
   return PEPS_OK;
@@ -2983,7 +2993,7 @@ int peps_group_create(peps_ctx* const* ctxs, int n, peps_group** out) {
   if (e == cudaSuccess) e = galloc(&G->d_flops, sizeof(double));
   if (e == cudaSuccess) e = galloc(&G->d_jsw, sizeof(unsigned long long));
   if (e == cudaSuccess)
-    e = cudaMemcpy(G->d_items, items.data(), items.size() * sizeof(GroupItem), cudaMemcpyHostToDevice);
+    e = upload(G->ctxs[0]->stream, G->d_items, items.data(), items.size() * sizeof(GroupItem));
   if (e == cudaSuccess && G->smem > 48 * 1024)
     e = G->f64 ? cudaFuncSetAttribute(k_eval_group<double, SAMPLE_THREADS>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024)
                : cudaFuncSetAttribute(k_eval_group<float, SAMPLE_THREADS>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
@@ -3212,9 +3222,9 @@ extern "C" int peps_selftest_tc_timeout(void) {
   if (cudaMalloc(&dA, A.size() * 4) != cudaSuccess || cudaMalloc(&dB, B.size() * 4) != cudaSuccess ||
       cudaMalloc(&dC, Cg.size() * 4) != cudaSuccess || cudaMalloc(&derr, sizeof(int)) != cudaSuccess)
     return done(PEPS_ENOMEM);
-  cudaMemcpy(dA, A.data(), A.size() * 4, cudaMemcpyHostToDevice);
-  cudaMemcpy(dB, B.data(), B.size() * 4, cudaMemcpyHostToDevice);
-  cudaMemset(derr, 0, sizeof(int));
+  upload(st, dA, A.data(), A.size() * 4);
+  upload(st, dB, B.data(), B.size() * 4);
+  cudaMemsetAsync(derr, 0, sizeof(int), st);
   int dev = 0, sms = 152;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -3235,7 +3245,7 @@ extern "C" int peps_selftest_tc_timeout(void) {
     if (cudaStreamSynchronize(st) != cudaSuccess || cudaGetLastError() != cudaSuccess) return done(PEPS_ECUDA);
     int h = -1;
     cudaMemcpy(&h, derr, sizeof(int), cudaMemcpyDeviceToHost);
-    cudaMemset(derr, 0, sizeof(int));
+    cudaMemsetAsync(derr, 0, sizeof(int), st);
     // the withheld MMAs must be noticed (with no MMA issued the grace wait runs out too,
     // so bit 2 is set as well)
     if (pass == 0 && h != 3) rc = PEPS_ESTATE;
