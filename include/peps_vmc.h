@@ -307,7 +307,8 @@ int peps_set_trunc_fp64(peps_ctx* ctx, int enable);
 /* CUDA graphs for the batched engine (enable = 1; 0 = direct launches, the default): the
  * launch sequence of a Metropolis sweep (per exponent p) and of an evaluation of the chains
  * (per use of the sweep's cached environments) is captured into a graph on first use and
- * replayed on later calls, one graph per chunk of chains; the sweep number reaches the
+ * replayed on later calls with the same number of configurations and the same arrays, one graph
+ * per chunk of chains (at most 64 are kept, the last used ones); the sweep number reaches the
  * kernels through device memory, so replays draw the same random numbers as direct launches
  * and every result is the same bits.  Replays skip the host's per-launch work, which counts
  * for small problems.  Per-launch profiling (peps_profile) and autotuning run without them;

@@ -329,15 +329,27 @@ struct BatchImpl : BatchIface {
   double *es_tmp = nullptr, *ea_tmp = nullptr;
   uint32_t* d_sweep = nullptr;   // the sweep number the accept kernels read
   double* jflops_dev = nullptr;  // Jacobi flop counter, fed while per-launch profiling is on
-  // CUDA graphs: one captured launch sequence per (operation, exponent or cache use, chunk,
-  // buffers), replayed on later calls; its flops and launch count are those of the capture
+  // CUDA graphs: one captured launch sequence per key, replayed on later calls; its flops and
+  // launch count are those of the capture.  The key holds all that a capture bakes in and a later
+  // call may change: operation, exponent or cache use, first chain, number of chains, and every
+  // array of the caller.  At most GRAPHS_MAX are kept (a cooling step of a chunked context takes
+  // three per chunk); the one unused for longest goes first.
   struct Graph {
     cudaGraphExec_t exec = nullptr;
     double flops = 0;
-    long long launches = 0;
+    long long launches = 0, used = 0;
   };
+  typedef std::array<long long, 10> GraphKey;
+  static constexpr size_t GRAPHS_MAX = 64;
   bool graphs = false;
-  std::map<std::tuple<int, int, long long, const void*, const void*>, Graph> gcache;
+  std::map<GraphKey, Graph> gcache;
+  long long guse = 0;
+  static GraphKey graph_key(int op, int opt, int off, int n, std::initializer_list<const void*> arrays) {
+    GraphKey k{op, opt, off, n};
+    size_t i = 4;
+    for (const void* a : arrays) k[i++] = (long long)(uintptr_t)a;
+    return k;
+  }
   // Chain programs (pv_prog.cuh) by (sequence, options, chains per SM), and the site tensors
   // they were recorded with
   enum { SEQ_EVAL, SEQ_MC, SEQ_DOWN, SEQ_DRAW, SEQ_AMP, SEQ_OROWS };
@@ -509,7 +521,7 @@ struct BatchImpl : BatchIface {
   // Runs fn's launch sequence on the engine's stream: directly, or (graphs on, no per-launch
   // profiling) from a graph captured on first use.  A capture that fails leaves graphs off.
   template <typename F>
-  void launch(const std::tuple<int, int, long long, const void*, const void*>& key, F&& fn) {
+  void launch(const GraphKey& key, F&& fn) {
     if (!graphs || (be.prof && be.prof->on)) {
       fn();
       return;
@@ -541,10 +553,18 @@ struct BatchImpl : BatchIface {
       }
       rec.flops = run.flops - f0;
       rec.launches = be.prof ? be.prof->launches - l0 : 0;
+      if (gcache.size() >= GRAPHS_MAX) {
+        auto old = gcache.begin();
+        for (auto k = gcache.begin(); k != gcache.end(); ++k)
+          if (k->second.used < old->second.used) old = k;
+        cudaGraphExecDestroy(old->second.exec);
+        gcache.erase(old);
+      }
       it = gcache.emplace(key, rec).first;
       run.flops = f0;
       if (be.prof) be.prof->launches = l0;
     }
+    it->second.used = ++guse;
     cudaGraphLaunch(it->second.exec, be.st);
     run.flops += it->second.flops;
     if (be.prof) be.prof->launches += it->second.launches;
@@ -576,7 +596,7 @@ struct BatchImpl : BatchIface {
       a.slot[PS_ES] = es0;
       a.slot[PS_EA] = ea0;
       a.slot[PS_O] = O0;
-      launch(std::make_tuple(0, cu ? 1 : 0, (long long)off, (const void*)S, (const void*)O),
+      launch(graph_key(0, cu ? 1 : 0, off, n, {S0, la0, sg0, es0, ea0, O0}),
              [&]() {
                if (p) exec(p, a);
                else run.eval(S0, n, la0, sg0, es0, ea0, O0, No, cu);
@@ -604,7 +624,7 @@ struct BatchImpl : BatchIface {
       for (int k = 0; k < n_sweeps; ++k) {
         k_set_sweep<<<1, 1, 0, be.st>>>(d_sweep, (uint32_t)(sweep0 + k));
         if (be.prof) be.prof->launches += 1;
-        launch(std::make_tuple(1, p, (long long)off, (const void*)S, (const void*)acc), [&]() {
+        launch(graph_key(1, p, off, n, {S0, acc, prop}), [&]() {
           if (pr) exec(pr, a);
           else run.mc(S0, n, p, seed, off, (uint32_t)(sweep0 + k), acc + off, prop + off);
         });
