@@ -368,7 +368,7 @@ struct OpTrunc {
       W sj = sig[j];
       for (int i = 0; i < nc; ++i) {
         W si = sig[i];
-        rank += (si > sj || (si == sj && i < j)) ? 1 : 0;
+        rank += sv_before(si, i, sj, j) ? 1 : 0;
       }
       order[rank] = j;
     }

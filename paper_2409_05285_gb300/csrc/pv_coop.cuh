@@ -90,6 +90,16 @@ PV_HD T cta_max(T v, T* red) {
 #endif
 }
 
+// Whether column i of norm a comes before column j of norm b in the descending order of singular
+// values (ties by index).  A norm that is not a number comes last, so the ranks are a permutation
+// for any input: they index the kept vectors.
+template <typename T>
+PV_HD bool sv_before(T a, int i, T b, int j) {
+  a = a == a ? a : (T)-1;
+  b = b == b ? b : (T)-1;
+  return a > b || (a == b && i < j);
+}
+
 // ---------------------------------------------------------------------------------------
 // A small einsum: out[o...] = sum_k A[..] * B[..] with single-letter labels.  Operands
 // are dense row-major in their label order; `dims` maps 'a'..'z' to extents.

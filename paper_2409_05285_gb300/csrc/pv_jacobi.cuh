@@ -370,7 +370,7 @@ __device__ __forceinline__ void jac_matrix(const OpTrunc<ST>& op, int s, unsigne
       const T sj = sig[j];
       for (int i = 0; i < nc; ++i) {
         const T si = sig[i];
-        rank += (si > sj || (si == sj && i < j)) ? 1 : 0;
+        rank += sv_before(si, i, sj, j) ? 1 : 0;
       }
       order[rank] = j;
     }

@@ -339,7 +339,7 @@ PV_HDN double compress(const Geom& g, Scratch<T>& sc, Shared<T>& sh, int p, cons
       T sj = sc.sig[j];
       for (int i = 0; i < nc; ++i) {
         T si = sc.sig[i];
-        rank += (si > sj || (si == sj && i < j)) ? 1 : 0;
+        rank += sv_before(si, i, sj, j) ? 1 : 0;
       }
       sc.order[rank] = j;
     }

@@ -137,7 +137,7 @@ __device__ void su_jacobi_cols(const double* X, int rows, int cols, double* Y, d
   PV_SYNC();
   for (int j = PV_TID; j < cols; j += PV_NTHR) {
     int rank = 0;
-    for (int i = 0; i < cols; ++i) rank += (sig[i] > sig[j] || (sig[i] == sig[j] && i < j)) ? 1 : 0;
+    for (int i = 0; i < cols; ++i) rank += sv_before(sig[i], i, sig[j], j) ? 1 : 0;
     ord[rank] = j;
   }
   PV_SYNC();
