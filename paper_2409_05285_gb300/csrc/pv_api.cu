@@ -350,41 +350,51 @@ struct BatchImpl : BatchIface {
     for (const void* a : arrays) k[i++] = (long long)(uintptr_t)a;
     return k;
   }
-  // Chain programs (pv_prog.cuh) by (sequence, options, chains per SM), and the site tensors
-  // they were recorded with
+  // Chain programs (pv_prog.cuh).  What a sequence records depends on the number of chains through
+  // the block shape alone, that is through the chains per SM up to PG_PER_SM: a program is kept by
+  // (sequence, options, chains per SM, site tensors), and the figures that decide whether a call
+  // runs as one (pg_wins, for its own number of chains) by sequence.
   enum { SEQ_EVAL, SEQ_MC, SEQ_DOWN, SEQ_DRAW, SEQ_AMP, SEQ_OROWS };
+  struct Plan {
+    bool bad;   // an operation has no program form in any block
+    int nops;
+    double flops;
+    long long largest;
+    bool tc;
+  };
+  std::map<std::tuple<int, int, const void*>, Plan> plans;
   std::map<std::tuple<int, int, int, const void*>, PgProgram> progs;
+  size_t prog_bytes = 0;    // device bytes of all programs, at most pg_pool_bytes(N)
+  long long calls = 0;      // calls so far: a program used in the current one is not dropped
   BatchImpl() : run(be) {}
   ~BatchImpl() override {
     drop_graphs();
-    drop_programs();
+    for (auto& kv : progs) cudaFree(kv.second.d_ops);   // null where there is none
+  }
+  void drop_program(typename std::map<std::tuple<int, int, int, const void*>, PgProgram>::iterator it) {
+    if (it->second.size) {
+      cudaStreamSynchronize(be.st);   // launches of it may be queued
+      drop_graphs();                  // and captures hold its address
+      cudaFree(it->second.d_ops);
+      prog_bytes -= it->second.size;
+    }
+    progs.erase(it);
   }
   void drop_programs() {
-    for (auto& kv : progs) {
-      if (kv.second.d_ops) cudaFree(kv.second.d_ops);
-      if (kv.second.d_tab) cudaFree(kv.second.d_tab);
-    }
-    progs.clear();
+    while (!progs.empty()) drop_program(progs.begin());
+    plans.clear();
   }
   // The program of a sequence for n chains: recorded and uploaded on first use by fn, which
-  // issues the runner's operations for one chain on the arrays of `ext`.  Null where an
-  // operation has no program form (too large for a block's shared memory): batched launches
-  // then.
+  // issues the runner's operations for one chain on the arrays of `ext`.  Null where batched launches
+  // are the choice: the sequence is faster that way at n chains, an operation has no program form
+  // (too large for a block's shared memory), or there is no room.
   template <typename F>
   const PgProgram* program(int seq, int opt, int n, const std::vector<typename PgBuild<T>::Ext>& ext, F&& fn) {
     if (N > 256 || (be.prof && be.prof->on)) return nullptr;   // profiling times every launch
-    const int q = std::min((n + be.sms - 1) / be.sms, 16);   // block shapes depend on the chains per SM
-    const auto key = std::make_tuple(seq, opt, q < 16 ? q : n, (const void*)run.theta);
-    auto it = progs.find(key);
-    if (it != progs.end()) return it->second.bad ? nullptr : &it->second;
-    PgProgram pr;
-    const double f0 = run.flops;
-    // a first recording finds the largest operation; blocks whose shared memory it exceeds get a
-    // larger share
-    int threads = 512, per_sm = 1;
-    bool sized = false;
-    for (;;) {
-      PgBuild<T> bd;
+    PgBuild<T> bd;
+    double flops = 0;
+    auto record = [&](int threads, int per_sm) {
+      bd = PgBuild<T>();
       bd.per_sm = per_sm;
       bd.threads = threads;
       bd.budget = PG_SMEM / per_sm - PG_STATIC;
@@ -395,29 +405,45 @@ struct BatchImpl : BatchIface {
         bd.sc[k] = sc[k];
         bd.i8[k] = i8[k];
       }
+      const double f0 = run.flops;
       run.flops = 0;
       be.rec = &bd;
       fn();
       be.rec = nullptr;
-      pr.flops = run.flops;
+      flops = run.flops;
       run.flops = f0;
+    };
+    auto pl = plans.find(std::make_tuple(seq, opt, (const void*)run.theta));
+    bool whole = false;   // bd holds the record of blocks of a whole SM
+    if (pl == plans.end()) {
+      record(512, 1);
+      whole = true;
+      pl = plans.emplace(std::make_tuple(seq, opt, (const void*)run.theta),
+                         Plan{bd.bad, (int)bd.ops.size(), flops, bd.largest, bd.tc_used}).first;
+    }
+    const Plan& plan = pl->second;
+    if (plan.bad || !pg_wins(n, plan.nops, plan.flops, sizeof(T) == 8)) return nullptr;
+    const int q = std::min((n + be.sms - 1) / be.sms, PG_PER_SM);
+    const auto key = std::make_tuple(seq, opt, q, (const void*)run.theta);
+    auto it = progs.find(key);
+    if (it != progs.end()) {
+      it->second.used = calls;
+      return it->second.bad ? nullptr : &it->second;
+    }
+    // blocks whose shared memory the largest operation exceeds get a larger share
+    const int threads = pg_threads(n, be.sms, plan.largest, plan.tc);
+    int per_sm = std::min(512 / threads, q);
+    for (;;) {
+      if (!whole || threads != 512 || per_sm != 1) record(threads, per_sm);
+      if (!bd.bad || per_sm == 1) break;
+      per_sm = per_sm > 4 ? per_sm / 2 : per_sm - 1;
+    }
+    PgProgram pr;
+    pr.used = calls;
+    pr.bad = bd.bad;
+    if (!pr.bad) {
       pr.nops = (int)bd.ops.size();
-      if (!sized && !bd.bad) {
-        if (!pg_wins(n, pr.nops, pr.flops, sizeof(T) == 8)) {
-          pr.bad = true;
-          break;
-        }
-        sized = true;
-        threads = pg_threads(n, be.sms, bd.largest, bd.tc_used);
-        per_sm = std::min(512 / threads, q);
-        if (threads < 512) continue;
-      }
-      if (bd.bad && per_sm > 1) {
-        per_sm = per_sm > 4 ? per_sm / 2 : per_sm - 1;
-        continue;
-      }
-      pr.bad = bd.bad;
-      if (pr.bad) break;
+      pr.flops = flops;
       PgOp end;
       memset(&end, 0, sizeof(end));
       end.kind = -1;
@@ -428,23 +454,31 @@ struct BatchImpl : BatchIface {
       pr.arena = (bd.need + 127) & ~(size_t)127;
       pr.bytes = bd.bytes;
       const size_t ob = bd.ops.size() * sizeof(PgOp), tb = (bd.tab.size() + 4) * sizeof(int);
+      pr.size = ob + tb;
+      while (prog_bytes + pr.size > pg_pool_bytes(N)) {   // the one unused for longest makes room
+        auto old = progs.end();
+        for (auto k = progs.begin(); k != progs.end(); ++k)
+          if (k->second.size && k->second.used != calls && (old == progs.end() || k->second.used < old->second.used))
+            old = k;
+        if (old == progs.end()) return nullptr;
+        drop_program(old);
+      }
       // another thread may be capturing a stream of its own: an allocation here is no part of that
       cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
       cudaThreadExchangeStreamCaptureMode(&mode);
-      cudaError_t e = cudaMalloc((void**)&pr.d_ops, ob);
-      if (e == cudaSuccess) e = cudaMalloc((void**)&pr.d_tab, tb);
+      cudaError_t e = cudaMalloc((void**)&pr.d_ops, pr.size);
       cudaThreadExchangeStreamCaptureMode(&mode);
+      pr.d_tab = (int*)((char*)pr.d_ops + ob);
       if (e == cudaSuccess) e = upload(be.st, pr.d_ops, bd.ops.data(), ob);
       if (e == cudaSuccess) e = upload(be.st, pr.d_tab, bd.tab.data(), bd.tab.size() * sizeof(int));
       if (e != cudaSuccess) {
         if (pr.d_ops) cudaFree(pr.d_ops);
-        if (pr.d_tab) cudaFree(pr.d_tab);
         pr = PgProgram();
         pr.bad = true;
         if (e != cudaErrorMemoryAllocation) return nullptr;   // the caller reports the error
         cudaGetLastError();   // no room: the batched launches need none
       }
-      break;
+      prog_bytes += pr.size;
     }
     it = progs.emplace(key, pr).first;
     return pr.bad ? nullptr : &it->second;
@@ -469,6 +503,7 @@ struct BatchImpl : BatchIface {
 
   // log|rho| and signs (plain_amplitude) and O rows (plain_log_derivative) of n configurations
   void amplitude(const uint8_t* S, int n, double* la, int8_t* sg) {
+    ++calls;
     count_jacobi();
     const PgProgram* p = program(SEQ_AMP, 0, n, {slot(S, PS_S), slot(la, PS_LA), slot(sg, PS_SG)},
                                  [&]() { plain_amplitude(run, S, 1, la, sg); });
@@ -480,6 +515,7 @@ struct BatchImpl : BatchIface {
     exec(p, a);
   }
   void orows(const uint8_t* S, int n, T* O, long long No) {
+    ++calls;
     count_jacobi();
     const PgProgram* p = program(SEQ_OROWS, 0, n, {slot(S, PS_S), slot(O, PS_O)},
                                  [&]() { plain_log_derivative(run, S, 1, O, No); });
@@ -574,6 +610,7 @@ struct BatchImpl : BatchIface {
   void eval(const uint8_t* S, int nb, double* la, int8_t* sg, double* es, double* ea, void* O,
             bool cached) override {
     run.flops = 0;
+    ++calls;
     count_jacobi();
     for (int off = 0; off < nb; off += chunk) {
       int n = std::min(chunk, nb - off);
@@ -607,6 +644,7 @@ struct BatchImpl : BatchIface {
   void mc(uint8_t* S, int n_all, int p, uint64_t seed, long long sweep0, int n_sweeps, int* acc,
           int* prop) override {
     run.flops = 0;
+    ++calls;
     count_jacobi();
     run.sweep_dev = d_sweep;
     for (int off = 0; off < n_all; off += chunk) {
@@ -635,6 +673,7 @@ struct BatchImpl : BatchIface {
   void draw(uint8_t* S, int n_all, const double* u, double b_d, double expo,
             double* logq) override {
     run.flops = 0;
+    ++calls;
     count_jacobi();
     for (int off = 0; off < n_all; off += chunk) {
       const int n = std::min(chunk, n_all - off);
@@ -1327,7 +1366,7 @@ size_t peps_footprint(const peps_params* P) {
   }
   else b += (size_t)n * ((long long)P->L1 * P->L2 * sd.ENV * real + (long long)P->L1 * (P->L2 + 1) * 4);
   b += n * 8 * 3 + 6 * Np * 8 + (real == 4 ? Np * 4 : 0) + 2 * (size_t)nch * Np * 8;   // SR
-  if (batched) b += (size_t)N * 100 * 1024;   // chain programs: about 100 records a site and sequence
+  if (batched) b += pg_pool_bytes((int)N);
   return b + (1 << 20);
 }
 

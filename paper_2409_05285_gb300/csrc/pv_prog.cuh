@@ -12,7 +12,7 @@
 // truncations and dot products run the same per-matrix routines.
 //
 // A program is a list of PgOp records plus a pool of index tables in device memory, made once
-// per (sequence, block shape) and kept with the runner's work buffers.  Pointers to those
+// per (sequence, block shape) and kept with the runner's work buffers, up to pg_pool_bytes().  Pointers to those
 // buffers are absolute; the caller's arrays (configurations, outputs) are slots that every
 // launch binds anew.  Per-chain scalars and selections (val, num, den, val2; si, sj, valid,
 // accepted) and the chain's configuration live in shared memory.
@@ -98,8 +98,10 @@ static_assert(sizeof(PgOp) % 16 == 0, "16-byte copies");
 constexpr int PG_BLOCK = 8;          // operations fetched at a time
 
 struct PgProgram {
-  PgOp* d_ops = nullptr;             // device: nblk * PG_BLOCK records
-  int* d_tab = nullptr;
+  PgOp* d_ops = nullptr;             // device: nblk * PG_BLOCK records, then ...
+  int* d_tab = nullptr;              // ... the tables, `size` bytes together
+  size_t size = 0;
+  long long used = 0;                // the last call that ran it
   int nops = 0, threads = 0, per_sm = 0, tmem_cols = 0;
   size_t arena = 0;                  // dynamic shared memory of a block
   double flops = 0, bytes = 0;       // per chain
@@ -114,6 +116,12 @@ cudaError_t pg_setup();
 
 constexpr size_t PG_STATIC = 5 * 1024;        // PgShared and the system's share
 constexpr size_t PG_SMEM = 227 * 1024;
+constexpr int PG_PER_SM = 16;                 // most chains an SM holds: a warp each
+
+// Device bytes that the programs of one engine may take on a lattice of N sites.  The longest
+// sequence (an evaluation with J2) is 99 records of 176 bytes a site and up to 55 KB of tables, 17 KB
+// a site at 8x8 D=4 chi=16: room for fifteen of them.
+inline size_t pg_pool_bytes(int N) { return (size_t)N * 256 * 1024; }
 
 // Threads per block for n chains on `sms` SMs (one chain per block): the 512 threads that 128
 // registers allow an SM are shared among the chains it has, down to one warp each, but a chain
