@@ -164,7 +164,10 @@ int peps_step(peps_ctx* ctx, int n_sweeps, int p, double tau, double eps, int ma
  * Grassmann-ordered contraction, evaluated as a configuration sign times the boundary-MPS
  * contraction (bond chi) of 32 signed slices per site.  peps_famp_create builds an
  * evaluator for up to n_max configurations (EINVAL for sizes outside the peps_init limits,
- * ENOMEM); peps_famp_eval takes host theta and configurations [nb][L1*L2] (entries 0..15,
+ * ENOMEM); the first call that takes local energies without the strip forms enlarges its work
+ * buffers, where n_max leaves them smaller, to eight configurations per SM, at most the four
+ * per bond and configuration that a call contracts, 4 GiB and an eighth of the free memory
+ * (without the room they stay as they are).  peps_famp_eval takes host theta and configurations [nb][L1*L2] (entries 0..15,
  * EINVAL otherwise) and writes log|psi| and the sign (0 where psi = 0) to host arrays. */
 typedef struct peps_famp peps_famp;
 int peps_famp_create(int L1, int L2, int D, int chi, int n_max, int precision, void* stream,

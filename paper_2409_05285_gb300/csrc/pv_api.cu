@@ -2243,6 +2243,8 @@ struct peps_famp {
   long long n16 = 0;
   int n_max = 0;
   int piece = 0;           // configurations taken through the engine at a time (at least n_max)
+  bool grown = false;      // famp_grow() has been here
+  std::vector<void*> engine_allocs;   // the engine's buffers, the extended indices among them
   long long *d_toff16 = nullptr, *d_toff32 = nullptr;
   double* d_th16 = nullptr;
   void* d_th32 = nullptr;
@@ -2291,6 +2293,69 @@ struct peps_famp {
 };
 
 namespace {
+
+// The engine and the extended indices for n configurations at a time, in place of those there are.
+// On failure everything stays as it was.
+int famp_engine(peps_famp* f, int n) {
+  peps_ctx* c = f->c;
+  int dev = 0, sms = 152;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const size_t first = c->allocs.size();
+  const int n_old = c->P.n_chains;
+  c->P.n_chains = n;   // sizes the engine's buffers
+  uint8_t* S32 = nullptr;
+  int8_t* csign = nullptr;
+  std::unique_ptr<BatchIface> eng;
+  BatchImpl<double>* b64 = nullptr;
+  BatchImpl<float>* b32 = nullptr;
+  int rc = dalloc(c, &S32, (size_t)n * c->N);
+  if (rc == PEPS_OK) rc = dalloc(c, &csign, (size_t)n);
+  if (rc == PEPS_OK && fp64(c)) {
+    eng.reset(b64 = new BatchImpl<double>());
+    rc = init_runner_t<double>(c, sms, b64, c->P.D, (const double*)f->d_th32, f->toff32);
+  } else if (rc == PEPS_OK) {
+    eng.reset(b32 = new BatchImpl<float>());
+    rc = init_runner_t<float>(c, sms, b32, c->P.D, (const float*)f->d_th32, f->toff32);
+  }
+  cudaStreamSynchronize(c->stream);   // before any buffer goes
+  std::vector<void*> mine(c->allocs.begin() + first, c->allocs.end());
+  c->allocs.resize(first);
+  if (rc == PEPS_OK) {
+    c->batch = std::move(eng);
+    f->b64 = b64;
+    f->b32 = b32;
+    f->d_S32 = S32;
+    f->d_csign = csign;
+    f->piece = n;
+    mine.swap(f->engine_allocs);
+  } else {
+    c->P.n_chains = n_old;
+  }
+  for (void* q : mine) cudaFree(q);
+  return rc;
+}
+
+// A local energy takes up to four amplitudes per bond and configuration (about 120 at 6x6), all
+// independent, so the first call that needs them lets the engine hold eight configurations per SM
+// however few chains a call has: in pieces of 128 an SR step of 128 chains took 296 ms (one program
+// block per SM), in pieces of 1216 104.  The work buffers stay below 4 GiB and an eighth of the
+// free memory; where they cannot be had, the engine stays as it is.
+int famp_grow(peps_famp* f) {
+  if (f->grown) return PEPS_OK;
+  peps_ctx* c = f->c;
+  int dev = 0, sms = 152;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  size_t fr = 0, tot = 0;
+  cudaMemGetInfo(&fr, &tot);
+  const size_t cap = std::min<size_t>(fr / 8, (size_t)4 << 30);
+  const long long want = std::min({8LL * sms, f->x_cap, (long long)(cap / batched_chain_bytes(&c->P))});
+  f->grown = true;
+  if (want <= f->piece) return PEPS_OK;
+  const int rc = famp_engine(f, (int)want);
+  return rc == PEPS_ENOMEM ? PEPS_OK : rc;
+}
 
 // log|psi| and sign of `count` configurations already on the device (entries checked unless
 // `check` is off: the caller knows them valid): in pieces through the extended indices and the
@@ -2440,6 +2505,7 @@ int famp_energies(peps_famp* f, int nb, double t_hop, double U, double mu) {
   }
   PV_TRY(famp_amplitudes(f, f->d_S16, nb, f->d_la, f->d_sg));   // also checks the entries
   if (f->strips) return famp_strips(f, nb, FAMP_ELOC, 2, 0, 0, t_hop, U, mu);
+  PV_TRY(famp_grow(f));
   const unsigned gb = (unsigned)((nb + 127) / 128);
   PV_KLAUNCH(&c->kprof, st, "k_fhop_count", 0.0, 0.0,
              k_fhop_count<<<gb, 128, 0, st>>>(nb, N, f->d_S16, f->d_bi, f->d_bj, f->nbonds, f->d_cnt));
@@ -2599,27 +2665,12 @@ int peps_famp_create(int L1, int L2, int D, int chi, int n_max, int precision, v
     f->c = nullptr;
     return rc;
   };
-  int rc, dev = 0, sms = 152;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  // A local energy takes about 120 amplitudes per configuration (6x6), all independent, so the engine
-  // holds eight configurations per SM however few chains a call has: in pieces of 128 an SR step of
-  // 128 chains took 296 ms (one program block per SM), in pieces of 1216 104.  The larger work buffers stay below 4 GiB and an eighth of the free memory.
-  f->piece = n_max;
-  {
-    size_t fr = 0, tot = 0;
-    cudaMemGetInfo(&fr, &tot);
-    const size_t per = batched_chain_bytes(&c->P), cap = std::min<size_t>(fr / 8, (size_t)4 << 30);
-    f->piece = (int)std::max<long long>(n_max, std::min<long long>(8LL * sms, (long long)(cap / per)));
-  }
-  c->P.n_chains = f->piece;   // of the engine's buffers
+  int rc;
   if ((rc = dalloc(c, &f->d_toff16, (N + 1) * sizeof(long long)))) return bail(rc);
   if ((rc = dalloc(c, &f->d_toff32, (N + 1) * sizeof(long long)))) return bail(rc);
   if ((rc = dalloc(c, &f->d_th16, (size_t)f->n16 * sizeof(double)))) return bail(rc);
   if ((rc = dalloc(c, (unsigned char**)&f->d_th32, (size_t)f->toff32[N] * real))) return bail(rc);
   if ((rc = dalloc(c, &f->d_S16, (size_t)n_max * N))) return bail(rc);
-  if ((rc = dalloc(c, &f->d_S32, (size_t)f->piece * N))) return bail(rc);
-  if ((rc = dalloc(c, &f->d_csign, (size_t)f->piece))) return bail(rc);
   if ((rc = dalloc(c, &f->d_sg, (size_t)n_max))) return bail(rc);
   if ((rc = dalloc(c, &f->d_la, (size_t)n_max * sizeof(double)))) return bail(rc);
   if ((rc = dalloc(c, &f->d_bad, sizeof(int)))) return bail(rc);
@@ -2627,16 +2678,9 @@ int peps_famp_create(int L1, int L2, int D, int chi, int n_max, int precision, v
   if (upload(c->stream, f->d_toff16, f->toff16.data(), (N + 1) * sizeof(long long)) != cudaSuccess ||
       upload(c->stream, f->d_toff32, f->toff32.data(), (N + 1) * sizeof(long long)) != cudaSuccess)
     return bail(PEPS_ECUDA);
-  if (precision == PEPS_FP64) {
-    f->b64 = new BatchImpl<double>();
-    c->batch.reset(f->b64);
-    rc = init_runner_t<double>(c, sms, f->b64, D, (const double*)f->d_th32, f->toff32);
-  } else {
-    f->b32 = new BatchImpl<float>();
-    c->batch.reset(f->b32);
-    rc = init_runner_t<float>(c, sms, f->b32, D, (const float*)f->d_th32, f->toff32);
-  }
-  if (rc != PEPS_OK) return bail(rc);
+  if ((rc = dalloc(c, &c->d_jflops, sizeof(double)))) return bail(rc);   // outlives an engine
+  if (cudaMemsetAsync(c->d_jflops, 0, sizeof(double), c->stream) != cudaSuccess) return bail(PEPS_ECUDA);
+  if ((rc = famp_engine(f.get(), n_max))) return bail(rc);
   *out = f.release();
   return PEPS_OK;
 }
@@ -2960,7 +3004,11 @@ const char* peps_famp_last_error(const peps_famp* f) { return f && f->c ? f->c->
 
 void peps_famp_free(peps_famp* f) {
   if (!f) return;
-  if (f->c) peps_free(f->c);
+  if (f->c) {
+    if (f->c->stream) cudaStreamSynchronize(f->c->stream);
+    for (void* q : f->engine_allocs) cudaFree(q);
+    peps_free(f->c);
+  }
   delete f;
 }
 
