@@ -22,8 +22,8 @@
 //    per lane group and step;
 //  - c and s are broadcast back to the lane group; a step in which no pair rotates stores
 //    nothing.
-// Sums are the same trees as the butterfly's (addition commutes), so every bit is that of
-// jacobi().
+// Sums are the same trees as the butterfly's (addition commutes) and every product that enters one
+// is fused as there (jac_fma, jac_rot), so every bit is that of jacobi(), in float32 and float64.
 //
 // Measured (mean per launch over one evaluation, the former kernel in brackets): float32 8x8
 // D=4 chi=16, 2048 chains 0.51 ms (1.73); 6x6 D=4 chi=16, 128 chains 63 us (347); 10x10 D=6
@@ -122,6 +122,20 @@ __device__ __forceinline__ T jac_reduce(T (&v)[TT], int G, int gl) {
   }
 }
 
+// One term of a dot product or norm, and the rotation of one element of a pair, their rounding
+// pinned to that of jacobi().  Left to the compiler, which products of an unrolled sum are fused depends
+// on the variant below: in float64 the variants then differed from each other in the last bits
+// (2e-14 in the kept vectors of 64 x 64 matrices).
+__device__ __forceinline__ float jac_fma(float x, float y, float a) { return __fmaf_rn(x, y, a); }
+__device__ __forceinline__ double jac_fma(double x, double y, double a) { return __fma_rn(x, y, a); }
+__device__ __forceinline__ float jac_mul(float x, float y) { return __fmul_rn(x, y); }
+__device__ __forceinline__ double jac_mul(double x, double y) { return __dmul_rn(x, y); }
+template <typename T>
+__device__ __forceinline__ void jac_rot(T c, T s, T x, T y, T& u, T& w) {
+  u = jac_fma(c, x, -jac_mul(s, y));
+  w = jac_fma(s, x, jac_mul(c, y));
+}
+
 // Column pair of slot pr in round rnd of the round-robin order (p < q); false when the slot is
 // past the end or holds the empty position of an odd column count.
 __device__ __forceinline__ bool jac_pair(int rnd, int pr, int np, int nc, int& p, int& q) {
@@ -192,7 +206,7 @@ __device__ __forceinline__ void jac_matrix(const OpTrunc<ST>& op, int s, unsigne
         for (int j = 0; j < nc; ++j)
           for (int i = lane; i < len; i += 32) {
             const T y = Y[j * ldy + pos(i)];
-            nf2 += y * y;
+            nf2 = jac_fma(y, y, nf2);
           }
         nf2 = warp_sum(nf2);
         if (lane == 0) red[0] = nf2;
@@ -206,7 +220,7 @@ __device__ __forceinline__ void jac_matrix(const OpTrunc<ST>& op, int s, unsigne
             T u[VW];
             jac_ld<T, VW>(u, Y + (size_t)j * ldy + (c * G + gl) * VW);
 #pragma unroll
-            for (int k = 0; k < VW; ++k) a += u[k] * u[k];
+            for (int k = 0; k < VW; ++k) a = jac_fma(u[k], u[k], a);
           }
         for (int o = G >> 1; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
         if (j < nc && gl == 0) {
@@ -248,14 +262,14 @@ __device__ __forceinline__ void jac_matrix(const OpTrunc<ST>& op, int s, unsigne
                 for (int c = 0; c < CH; ++c)
                   if (c < chY)
 #pragma unroll
-                    for (int k = 0; k < VW; ++k) g[t] += x[t][c * VW + k] * y[t][c * VW + k];
+                    for (int k = 0; k < VW; ++k) g[t] = jac_fma(x[t][c * VW + k], y[t][c * VW + k], g[t]);
               } else {
                 for (int c = 0; c < chY; ++c) {
                   T u[VW], w[VW];
                   jac_ld<T, VW>(u, Y + xp[t] + c * G * VW);
                   jac_ld<T, VW>(w, Y + xq[t] + c * G * VW);
 #pragma unroll
-                  for (int k = 0; k < VW; ++k) g[t] += u[k] * w[k];
+                  for (int k = 0; k < VW; ++k) g[t] = jac_fma(u[k], w[k], g[t]);
                 }
               }
             }
@@ -295,10 +309,9 @@ __device__ __forceinline__ void jac_matrix(const OpTrunc<ST>& op, int s, unsigne
 #pragma unroll
                       for (int k = 0; k < VW; ++k) {
                         const T x0 = x[t][c * VW + k], y0 = y[t][c * VW + k];
-                        u[k] = c0 * x0 - s0 * y0;
-                        w[k] = s0 * x0 + c0 * y0;
-                        na[t] += u[k] * u[k];
-                        nb[t] += w[k] * w[k];
+                        jac_rot(c0, s0, x0, y0, u[k], w[k]);
+                        na[t] = jac_fma(u[k], u[k], na[t]);
+                        nb[t] = jac_fma(w[k], w[k], nb[t]);
                       }
                       jac_st<T, VW>(Y + xp[t] + c * G * VW, u);
                       jac_st<T, VW>(Y + xq[t] + c * G * VW, w);
@@ -311,10 +324,9 @@ __device__ __forceinline__ void jac_matrix(const OpTrunc<ST>& op, int s, unsigne
 #pragma unroll
                     for (int k = 0; k < VW; ++k) {
                       const T x0 = u[k], y0 = w[k];
-                      u[k] = c0 * x0 - s0 * y0;
-                      w[k] = s0 * x0 + c0 * y0;
-                      na[t] += u[k] * u[k];
-                      nb[t] += w[k] * w[k];
+                      jac_rot(c0, s0, x0, y0, u[k], w[k]);
+                      na[t] = jac_fma(u[k], u[k], na[t]);
+                      nb[t] = jac_fma(w[k], w[k], nb[t]);
                     }
                     jac_st<T, VW>(Y + xp[t] + c * G * VW, u);
                     jac_st<T, VW>(Y + xq[t] + c * G * VW, w);
@@ -330,8 +342,7 @@ __device__ __forceinline__ void jac_matrix(const OpTrunc<ST>& op, int s, unsigne
 #pragma unroll
                     for (int k = 0; k < VW; ++k) {
                       const T x0 = u[k], y0 = w[k];
-                      u[k] = c0 * x0 - s0 * y0;
-                      w[k] = s0 * x0 + c0 * y0;
+                      jac_rot(c0, s0, x0, y0, u[k], w[k]);
                     }
                     jac_st<T, VW>(vp + c * G * VW, u);
                     jac_st<T, VW>(vq + c * G * VW, w);
