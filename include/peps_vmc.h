@@ -374,8 +374,9 @@ int peps_last_counters(peps_ctx* ctx, double* flops, int64_t* jacobi_sweeps);
 long long peps_launches(const peps_ctx* ctx);
 
 /* Autotuner of the batched engine's launch shapes, keyed on the problem geometry (d^2 = 4,
- * D, chi, L1, L2, precision).  peps_autotune times `reps` evaluations of (at most 8192 of)
- * the context's chains per candidate (coordinate descent over the tensor-core grid size, the
+ * D, chi, L1, L2, precision).  The shapes are those of calls that launch their operations one by
+ * one; smaller calls run as one kernel, which has none of them.  peps_autotune times `reps`
+ * launched evaluations of (at most 8192 of) the context's chains per candidate (coordinate descent over the tensor-core grid size, the
  * contraction chunk, the chains per FFMA block and the truncation's threads; only the last two
  * without tensor cores) and keeps the fastest; the choice is stored in a process-wide table that later
  * contexts of the same geometry start from.  No candidate changes any result.  reps = 0
@@ -387,7 +388,8 @@ typedef struct {
   int grid_pct;    /* persistent tensor-core grid, per cent of the resident CTAs */
   int db_bytes;    /* kept for saved shapes; no effect */
   int ffma_g;      /* most chains per block of the FFMA contraction kernel */
-  int kc_max;      /* largest contraction chunk of the tensor-core kernel (8, 16, ..., 64) */
+  int kc_max;      /* largest contraction chunk of the tensor-core kernel (8, 16, ..., 64; it takes
+                      chunks of 8, 16 and 32) */
   double ms_before, ms_after;
   int pipelined;   /* kept for saved shapes; no effect */
   int stage_kb;    /* kept for saved shapes; no effect (32..200; 0 in peps_set_tune keeps the

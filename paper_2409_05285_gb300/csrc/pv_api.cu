@@ -305,6 +305,7 @@ struct BatchIface {
   virtual bool graphs_on() const = 0;
   virtual int graphs_captured() const = 0;
   virtual void drop_graphs() = 0;         // launch shapes changed: recapture on next use
+  virtual void set_programs(bool on) = 0; // off: every call launches its operations
   // float engines: truncate with a float64 working copy (g64: its global work area, or null)
   virtual bool set_trunc64(bool on, double* g64) = 0;
   virtual long long trunc_cap() const = 0;
@@ -364,6 +365,7 @@ struct BatchImpl : BatchIface {
   };
   std::map<std::tuple<int, int, const void*>, Plan> plans;
   std::map<std::tuple<int, int, int, const void*>, PgProgram> progs;
+  bool programs = true;
   size_t prog_bytes = 0;    // device bytes of all programs, at most pg_pool_bytes(N)
   long long calls = 0;      // calls so far: a program used in the current one is not dropped
   BatchImpl() : run(be) {}
@@ -390,7 +392,7 @@ struct BatchImpl : BatchIface {
   // (too large for a block's shared memory), or there is no room.
   template <typename F>
   const PgProgram* program(int seq, int opt, int n, const std::vector<typename PgBuild<T>::Ext>& ext, F&& fn) {
-    if (N > 256 || (be.prof && be.prof->on)) return nullptr;   // profiling times every launch
+    if (!programs || N > 256 || (be.prof && be.prof->on)) return nullptr;   // profiling times every launch
     PgBuild<T> bd;
     double flops = 0;
     auto record = [&](int threads, int per_sm) {
@@ -533,6 +535,7 @@ struct BatchImpl : BatchIface {
     graphs = on;
   }
   bool graphs_on() const override { return graphs; }
+  void set_programs(bool on) override { programs = on; }
   int graphs_captured() const override { return (int)gcache.size(); }
   bool set_trunc64(bool on, double* g64) override {
     if constexpr (std::is_same<T, float>::value) {
@@ -1867,13 +1870,19 @@ int peps_autotune(peps_ctx* c, int reps, peps_tune* out) {
   if (!c->batch) return fail(c, PEPS_ESTATE, "autotune: only the batched engine has launch shapes to tune");
   BatchTune& tu = c->batch->tuning();
   // every candidate is timed with direct launches (a graph would replay the shapes it was
-  // captured with)
+  // captured with, and a chain program has none of them: the shapes serve the calls that launch)
   const bool had_graphs = c->batch->graphs_on();
-  c->batch->set_graphs(false);
+  if (reps > 0) {
+    c->batch->set_graphs(false);
+    c->batch->set_programs(false);
+  }
   struct Restore {
     peps_ctx* c;
     bool on;
-    ~Restore() { c->batch->set_graphs(on); }
+    ~Restore() {
+      c->batch->set_graphs(on);
+      c->batch->set_programs(true);
+    }
   } restore{c, had_graphs};
   // time on at most 8192 chains: the best shapes depend on the chain count (a 2048-chain
   // subset picked one chain per FFMA block, which is slower at 8192 chains)
@@ -1900,25 +1909,26 @@ int peps_autotune(peps_ctx* c, int reps, peps_tune* out) {
   };
   double before = 0, cur = 0;
   if (reps > 0) {
+    // untimed: the first evaluation loads kernels
+    PV_TRY(launch_eval(c, c->d_S, n, c->d_log_abs, c->d_sign, c->d_es, c->d_ea, c->d_O, false));
     PV_TRY(timed(&before));
     cur = before;
-    // coordinate descent over the launch-shape parameters (results are the same for all)
-    const int grid_c[] = {50, 100, 200}, kc_c[] = {16, 32, 64}, g_c[] = {1, 16, 256}, tt_c[] = {32, 64, 256};
+    // coordinate descent over the launch-shape parameters (results are the same for all); chunks
+    // above 32 are the same kernels
+    const std::vector<int> cands[] = {{50, 100, 200}, {16, 64}, {1, 16, 256}, {32, 64, 256}};
     int* fields[] = {&tu.grid_pct, &tu.kc_max, &tu.ffma_g, &tu.trunc_threads};
-    const int* cands[] = {grid_c, kc_c, g_c, tt_c};
     for (int knob = c->batch->uses_tensor_cores() ? 0 : 2; knob < 4; ++knob) {
       int* field = fields[knob];
-      const int* cand = cands[knob];
       int best_v = *field;
-      for (int i = 0; i < 3; ++i) {
-        if (cand[i] == best_v) continue;
+      for (const int cand : cands[knob]) {
+        if (cand == best_v) continue;
         const int keep = *field;
-        *field = cand[i];
+        *field = cand;
         double ms = 0;
         PV_TRY(timed(&ms));
         if (ms < cur * 0.99) {
           cur = ms;
-          best_v = cand[i];
+          best_v = cand;
         } else {
           *field = keep;
         }
