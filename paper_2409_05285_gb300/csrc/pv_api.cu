@@ -956,10 +956,12 @@ int init_runner_t(peps_ctx* c, int sms, BatchImpl<T>* b, int Dn, const T* theta,
   const long long cap = 2 * cD * (cD + 1);
   const size_t trunc_bytes = (size_t)cap * sizeof(T) + (size_t)(cD + 4) * (sizeof(T) + 4) + 16;
   const bool trunc_global = trunc_bytes > 200 * 1024;   // room for Jacobi matrices in global memory
-  {
+  if (!pg_is_set_up<T>()) {   // the executor's limit is the last one set, and only here
     cudaError_t e = jac_setup<T, T>();
-    if constexpr (std::is_same<T, float>::value)
+    if constexpr (std::is_same<T, float>::value) {
       if (e == cudaSuccess) e = jac_setup<double, float>();
+      if (e == cudaSuccess) e = tc_setup();
+    }
     if (e == cudaSuccess) e = pg_setup<T>();
     if (e != cudaSuccess) return fail(c, PEPS_ECUDA, std::string("cudaFuncSetAttribute: ") + cudaGetErrorString(e));
   }
@@ -1040,7 +1042,6 @@ int init_runner_t(peps_ctx* c, int sms, BatchImpl<T>* b, int Dn, const T* theta,
     // also takes the right factors from the Gram matrix
     if ((rc = dalloc(c, &b->be.tc_err, sizeof(int)))) return rc;
     cudaError_t e = cudaMemsetAsync(b->be.tc_err, 0, sizeof(int), c->stream);
-    if (e == cudaSuccess) e = tc_setup();
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(kb_chol<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     if (e != cudaSuccess) return fail(c, PEPS_ECUDA, std::string("tensor-core setup: ") + cudaGetErrorString(e));

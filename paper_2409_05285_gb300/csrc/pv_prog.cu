@@ -710,6 +710,14 @@ cudaError_t pg_setup() {
 }
 
 template <typename T>
+bool pg_is_set_up() {
+  cudaFuncAttributes a;
+  if (cudaFuncGetAttributes(&a, kb_prog<T>) == cudaSuccess) return a.maxDynamicSharedSizeBytes == (int)(PG_SMEM - 1024);
+  cudaGetLastError();
+  return false;
+}
+
+template <typename T>
 void pg_launch(const PgProgram& p, const PgArgs& a, T jtol, double jtol64, int max_sweeps, unsigned long long* sweeps,
                int* err, int sms, cudaStream_t st) {
   const int grid = a.n < sms * p.per_sm ? a.n : sms * p.per_sm;
@@ -719,6 +727,8 @@ void pg_launch(const PgProgram& p, const PgArgs& a, T jtol, double jtol64, int m
 
 template cudaError_t pg_setup<float>();
 template cudaError_t pg_setup<double>();
+template bool pg_is_set_up<float>();
+template bool pg_is_set_up<double>();
 template void pg_launch<float>(const PgProgram&, const PgArgs&, float, double, int, unsigned long long*, int*, int,
                                cudaStream_t);
 template void pg_launch<double>(const PgProgram&, const PgArgs&, double, double, int, unsigned long long*, int*, int,
