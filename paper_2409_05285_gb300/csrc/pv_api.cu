@@ -393,6 +393,22 @@ struct BatchImpl : BatchIface {
   template <typename F>
   const PgProgram* program(int seq, int opt, int n, const std::vector<typename PgBuild<T>::Ext>& ext, F&& fn) {
     if (!programs || N > 256 || (be.prof && be.prof->on)) return nullptr;   // profiling times every launch
+    const int q = std::min((n + be.sms - 1) / be.sms, PG_PER_SM);
+    const auto key = std::make_tuple(seq, opt, q, (const void*)run.theta);
+    auto pl = plans.find(std::make_tuple(seq, opt, (const void*)run.theta));
+    auto wins = [&]() {
+      const Plan& p = pl->second;
+      return !p.bad && pg_wins(n, p.nops, p.flops, sizeof(T) == 8);
+    };
+    auto it = progs.end();
+    if (pl != plans.end()) {
+      if (!wins()) return nullptr;
+      it = progs.find(key);
+      if (it != progs.end()) {
+        it->second.used = calls;
+        return it->second.bad ? nullptr : &it->second;
+      }
+    }
     PgBuild<T> bd;
     double flops = 0;
     auto record = [&](int threads, int per_sm) {
@@ -415,25 +431,16 @@ struct BatchImpl : BatchIface {
       flops = run.flops;
       run.flops = f0;
     };
-    auto pl = plans.find(std::make_tuple(seq, opt, (const void*)run.theta));
     bool whole = false;   // bd holds the record of blocks of a whole SM
     if (pl == plans.end()) {
       record(512, 1);
       whole = true;
       pl = plans.emplace(std::make_tuple(seq, opt, (const void*)run.theta),
                          Plan{bd.bad, (int)bd.ops.size(), flops, bd.largest, bd.tc_used}).first;
-    }
-    const Plan& plan = pl->second;
-    if (plan.bad || !pg_wins(n, plan.nops, plan.flops, sizeof(T) == 8)) return nullptr;
-    const int q = std::min((n + be.sms - 1) / be.sms, PG_PER_SM);
-    const auto key = std::make_tuple(seq, opt, q, (const void*)run.theta);
-    auto it = progs.find(key);
-    if (it != progs.end()) {
-      it->second.used = calls;
-      return it->second.bad ? nullptr : &it->second;
+      if (!wins()) return nullptr;
     }
     // blocks whose shared memory the largest operation exceeds get a larger share
-    const int threads = pg_threads(n, be.sms, plan.largest, plan.tc);
+    const int threads = pg_threads(n, be.sms, pl->second.largest, pl->second.tc);
     int per_sm = std::min(512 / threads, q);
     for (;;) {
       if (!whole || threads != 512 || per_sm != 1) record(threads, per_sm);
