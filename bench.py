@@ -56,26 +56,26 @@ TF32_OVER_BF16 = 1.1 / 2.25
 # reports null.
 NCU_TRAFFIC = {
     ("heis8", "tf32", "kb_gemm_tc"): {
-        "chains": 2048,
+        "chains": 1024,
         "launches": 100,
-        "dram_bytes": 6969.22e6,        # DRAM read + write of the first 100 launches of the step
-        "alg_bytes": 9975.38e6,         # algorithmic bytes of the same 100 launches
-        "sources_sha256": "e7997e742bd0251c6223b3b09e0e0ea0a5c7b20f11f5fde0f50bb44526b564b0",
+        "dram_bytes": 2767.20e6,        # DRAM read + write of the first 100 launches of the step
+        "alg_bytes": 4987.76e6,         # algorithmic bytes of the same 100 launches
+        "sources_sha256": "e5743502f377395e704b2da11e6a8c16c421d34472b06e35d8db68a9f82bc66d",
         "source": "ncu --profile-from-start off --clock-control none --metrics "
                   "dram__bytes_read.sum,dram__bytes_write.sum,gpu__time_duration.sum "
                   "-k regex:kb_gemm_tc -c 100 (cold cache): the first 100 launches of the timed "
-                  "step at 2048 chains (shapes 100,12288,16,16,0), scaled by algorithmic bytes",
+                  "step at 1024 chains (default shapes, no autotune), scaled by algorithmic bytes",
     },
     ("j1j2_10", "tf32", "kb_gemm_tc"): {
-        "chains": 512,
+        "chains": 256,
         "launches": 100,
-        "dram_bytes": 38160.7e6,
-        "alg_bytes": 41258.7e6,
-        "sources_sha256": "e7997e742bd0251c6223b3b09e0e0ea0a5c7b20f11f5fde0f50bb44526b564b0",
+        "dram_bytes": 16398.6e6,
+        "alg_bytes": 19618.9e6,
+        "sources_sha256": "e5743502f377395e704b2da11e6a8c16c421d34472b06e35d8db68a9f82bc66d",
         "source": "ncu --profile-from-start off --clock-control none --metrics "
                   "dram__bytes_read.sum,dram__bytes_write.sum,gpu__time_duration.sum "
-                  "-k regex:^kb_gemm_tc$ -c 100 (cold cache): the first 100 launches of the timed "
-                  "step at 512 chains (default shapes, no autotune), scaled by algorithmic bytes",
+                  "-k regex:kb_gemm_tc -c 100 (cold cache): the first 100 launches of the timed "
+                  "step at 256 chains (default shapes, no autotune), scaled by algorithmic bytes",
     },
 }
 TRAFFIC_SOURCES = ("paper_2409_05285_gb300/csrc/pv_tc.cuh", "paper_2409_05285_gb300/csrc/pv_gemm.cuh",

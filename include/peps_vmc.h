@@ -330,7 +330,8 @@ int peps_graphs_captured(const peps_ctx* ctx);
  * copy of float32 O rows made once per step (no float64 issue spent on widening in the
  * passes; n_chains x N_o doubles, ENOMEM from peps_sr_step when they cannot be allocated);
  * 0 (default) = 3 where the rows are float32 in 16-byte site slices and the copy fits, else
- * 2 (the fused form was measured slower on GB300 at 8x8 and 10x10: float64 FMA issue bounds
+ * 2, as one cooperative kernel for the whole CG loop where N_p <= 4096 and n_chains x N_o <= 4e6
+ * (the same bits) (the fused form was measured slower on GB300 at 8x8 and 10x10: float64 FMA issue bounds
  * both forms, and it adds a grid barrier per chunk).  Every choice uses float64 products
  * and fixed summation orders; 2 and 3 give the same bits, the others agree to rounding.
  * EINVAL for other modes. */

@@ -1783,8 +1783,9 @@ __global__ void __launch_bounds__(256) kb_dot(OpDot<T> op, int n, ChainList cl) 
 
 // The same sums (lane l of one warp adds the entries l, l + 32, ... in order) of long vectors of few
 // chains: a block per chain, whose eight warps load 2048 entries ahead of the one that adds.
-// One warp alone waits for memory at every few entries: 46656 entries of 192 chains 73 us (10x10
-// D=6 chi=36), 8192 chains of 4096 are bound by memory either way.
+// One warp alone waits for memory at every few entries.  Measured out of a cold L2, a warp / a block:
+// 46656 entries of 192 chains (10x10 D=6 chi=36) 207 / 31 us, 4096 entries of 192 chains 21 / 8, of
+// 2048 chains 29 / 21, of 8192 chains (bound by memory either way) 63 / 58.
 constexpr int DOT_TILE = 2048;
 template <typename T>
 __global__ void __launch_bounds__(256) kb_dot_block(OpDot<T> op, int n, ChainList cl) {
