@@ -58,9 +58,9 @@ NCU_TRAFFIC = {
     ("heis8", "tf32", "kb_gemm_tc"): {
         "chains": 1024,
         "launches": 100,
-        "dram_bytes": 2767.20e6,        # DRAM read + write of the first 100 launches of the step
+        "dram_bytes": 2760.21e6,        # DRAM read + write of the first 100 launches of the step
         "alg_bytes": 4987.76e6,         # algorithmic bytes of the same 100 launches
-        "sources_sha256": "e5743502f377395e704b2da11e6a8c16c421d34472b06e35d8db68a9f82bc66d",
+        "sources_sha256": "3f344cdcf150e5a5dbe341992e0634d46ae1c2cd0d8791c9d7d2bf031ed7466d",
         "source": "ncu --profile-from-start off --clock-control none --metrics "
                   "dram__bytes_read.sum,dram__bytes_write.sum,gpu__time_duration.sum "
                   "-k regex:kb_gemm_tc -c 100 (cold cache): the first 100 launches of the timed "
@@ -69,9 +69,9 @@ NCU_TRAFFIC = {
     ("j1j2_10", "tf32", "kb_gemm_tc"): {
         "chains": 256,
         "launches": 100,
-        "dram_bytes": 16398.6e6,
+        "dram_bytes": 16400.0e6,
         "alg_bytes": 19618.9e6,
-        "sources_sha256": "e5743502f377395e704b2da11e6a8c16c421d34472b06e35d8db68a9f82bc66d",
+        "sources_sha256": "3f344cdcf150e5a5dbe341992e0634d46ae1c2cd0d8791c9d7d2bf031ed7466d",
         "source": "ncu --profile-from-start off --clock-control none --metrics "
                   "dram__bytes_read.sum,dram__bytes_write.sum,gpu__time_duration.sum "
                   "-k regex:kb_gemm_tc -c 100 (cold cache): the first 100 launches of the timed "

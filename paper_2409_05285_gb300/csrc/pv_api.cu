@@ -963,15 +963,6 @@ int init_runner_t(peps_ctx* c, int sms, BatchImpl<T>* b, int Dn, const T* theta,
   const long long cap = 2 * cD * (cD + 1);
   const size_t trunc_bytes = (size_t)cap * sizeof(T) + (size_t)(cD + 4) * (sizeof(T) + 4) + 16;
   const bool trunc_global = trunc_bytes > 200 * 1024;   // room for Jacobi matrices in global memory
-  if (!pg_is_set_up<T>()) {   // the executor's limit is the last one set, and only here
-    cudaError_t e = jac_setup<T, T>();
-    if constexpr (std::is_same<T, float>::value) {
-      if (e == cudaSuccess) e = jac_setup<double, float>();
-      if (e == cudaSuccess) e = tc_setup();
-    }
-    if (e == cudaSuccess) e = pg_setup<T>();
-    if (e != cudaSuccess) return fail(c, PEPS_ECUDA, std::string("cudaFuncSetAttribute: ") + cudaGetErrorString(e));
-  }
   std::vector<long long> sz;
   long long n8, nd;
   BatchBufs<T>::sizes(P->L1, P->L2, Dn, P->chi, sz, n8, nd);

@@ -2059,7 +2059,7 @@ struct CudaBE {
         t.sym = tc_symmetric(t, op_same(A, B)) ? 1 : 0;
         tc_shape(t, tune.kc_max);
         const size_t bytes = tc_smem_bytes(t);
-        if (bytes <= 200 * 1024) {   // what the kernels are configured for
+        if (bytes <= TC_SMEM_MAX) {
           // persistent grid of the CTAs that can be resident at once
           auto go = [&](auto kern, int by_regs) {
             const int tilesM = (t.M + TC_ROWS - 1) / TC_ROWS, tilesN = (t.N + t.TN - 1) / t.TN;
@@ -2069,6 +2069,7 @@ struct CudaBE {
             gy = gy < 1 ? 1 : (gy > n ? n : gy);
             gy = gy > 65535 ? 65535 : gy;
             dim3 gr(tilesM * tilesN, (unsigned)gy);
+            smem_cap(kern, bytes, TC_SMEM_MAX);
             PV_KLAUNCH(prof, st, "kb_gemm_tc", ein_bytes(raw, A, B, nw), 2.0 * raw.total * raw.kprod * nw,
                        pdl_if(early, kern, gr, TC_THREADS, bytes, st, t, out, os, swap ? B : A, swap ? A : B, n, tilesN, tc_err,
                                                            act));

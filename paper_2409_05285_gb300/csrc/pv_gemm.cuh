@@ -293,6 +293,7 @@ __global__ void __launch_bounds__(TC_THREADS, MINB) kb_gemm_tc(TcSpec t, float* 
 }
 
 // f(kernel, resident CTAs per SM that its registers allow) for the variant of a spec.
+constexpr int TC_SMEM_MAX = 200 * 1024;   // most dynamic shared memory of the kernels
 template <int NA, int NB, int MINB, typename F>
 void tc_modes(int mp, int mq, F&& f) {
   auto q = [&](auto MP) {
@@ -310,22 +311,6 @@ void tc_kernel(const TcSpec& t, F&& f) {
   else if (t.TN <= 128) tc_modes<4, 4, 5>(t.modeP, t.modeQ, f);
   else tc_modes<4, 8, 4>(t.modeP, t.modeQ, f);
 }
-// Shared memory of every variant.
-inline cudaError_t tc_setup() {
-  cudaError_t e = cudaSuccess;
-  TcSpec t;
-  for (int v = 0; v < 27; ++v) {
-    t.Kc = v < 9 ? 32 : 16;
-    t.TN = v < 18 ? 128 : 256;
-    t.modeP = v / 3 % 3;
-    t.modeQ = v % 3;
-    tc_kernel(t, [&](auto k, int) {
-      if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    });
-  }
-  return e;
-}
-
 #endif  // __CUDACC__
 
 }  // namespace pv

@@ -439,24 +439,7 @@ __global__ void __launch_bounds__(MAXT, MAXT == 256 ? 2 : 1) kb_jac(OpTrunc<ST> 
   for (int s = blockIdx.x; s < n; s += gridDim.x) jac_matrix<T, ST, CH, TT>(op, s, dyn, red, G, lg, chY, chV, tol);
 }
 
-constexpr int JAC_SMEM_MAX = 220 * 1024;   // dynamic shared memory the kernels are configured for
-
-template <typename T, typename ST>
-inline cudaError_t jac_setup() {
-  cudaError_t e = cudaSuccess;
-  auto set = [&](const void* f) {
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, JAC_SMEM_MAX);
-  };
-  set((const void*)kb_jac<T, ST, 1, 4, 256>);
-  set((const void*)kb_jac<T, ST, 1, 1, 256>);
-  set((const void*)kb_jac<T, ST, 2, 4, 256>);
-  set((const void*)kb_jac<T, ST, 2, 1, 256>);
-  set((const void*)kb_jac<T, ST, 4, 2, 256>);
-  set((const void*)kb_jac<T, ST, 4, 1, 256>);
-  set((const void*)kb_jac<T, ST, 8, 1, 512>);
-  set((const void*)kb_jac<T, ST, 0, 1, 512>);
-  return e;
-}
+constexpr int JAC_SMEM_MAX = 220 * 1024;   // most dynamic shared memory of the kernels
 
 // Launches the truncation of n chains; `threads`: 0 chooses the block, else its size.  Blocks
 // of few warps that take TT pairs per lane group keep the scalar arithmetic and the barriers of
@@ -486,7 +469,10 @@ inline void jac_launch(const OpTrunc<ST>& op, int n, const JacShape& s, T tol, i
   int grid = sms * res;
   grid = n < grid ? n : grid;
   const int nt = 32 * W;
-  auto go = [&](auto kern) { kern<<<grid, nt, s.bytes, st>>>(op, n, s.G, s.lg, s.chY, s.chV, tol); };
+  auto go = [&](auto kern) {
+    smem_cap(kern, s.bytes, JAC_SMEM_MAX);
+    kern<<<grid, nt, s.bytes, st>>>(op, n, s.G, s.lg, s.chY, s.chV, tol);
+  };
   if (s.chY <= 1) {
     if (TT == 4) go(kb_jac<T, ST, 1, 4, 256>); else go(kb_jac<T, ST, 1, 1, 256>);
   } else if (s.chY <= 2) {

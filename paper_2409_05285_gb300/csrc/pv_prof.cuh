@@ -94,6 +94,15 @@ struct KProf {
 // block that took them first would wait for this kernel's end).  Launched without pdl() both do
 // nothing.
 #if defined(__CUDACC__)
+// Lets a kernel that is about to be launched with `bytes` of dynamic shared memory have more than the
+// default 48 KB (its static arrays, a few hundred bytes, included): up to `cap`, the same for every
+// caller, so that no context lowers it under another.  Set where the kernel is launched, since the
+// attribute loads the kernel's code: forty of them set by the first context took it 17 of 49 ms.
+template <typename K>
+inline void smem_cap(K kern, size_t bytes, int cap) {
+  if (bytes > 44 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, cap);
+}
+
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_go() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

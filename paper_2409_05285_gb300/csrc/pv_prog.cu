@@ -705,30 +705,15 @@ __global__ void __launch_bounds__(512, 1) kb_prog(const PgOp* __restrict__ ops, 
 }  // namespace
 
 template <typename T>
-cudaError_t pg_setup() {
-  return cudaFuncSetAttribute(kb_prog<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(PG_SMEM - 1024));
-}
-
-template <typename T>
-bool pg_is_set_up() {
-  cudaFuncAttributes a;
-  if (cudaFuncGetAttributes(&a, kb_prog<T>) == cudaSuccess) return a.maxDynamicSharedSizeBytes == (int)(PG_SMEM - 1024);
-  cudaGetLastError();
-  return false;
-}
-
-template <typename T>
 void pg_launch(const PgProgram& p, const PgArgs& a, T jtol, double jtol64, int max_sweeps, unsigned long long* sweeps,
                int* err, int sms, cudaStream_t st) {
   const int grid = a.n < sms * p.per_sm ? a.n : sms * p.per_sm;
-  kb_prog<T><<<grid, p.threads, pg_arena_off<T>() + p.arena, st>>>(p.d_ops, (p.nops + PG_BLOCK - 1) / PG_BLOCK, p.d_tab, a, p.tmem_cols,
+  const size_t smem = pg_arena_off<T>() + p.arena;
+  smem_cap(kb_prog<T>, smem, (int)(PG_SMEM - 1024));
+  kb_prog<T><<<grid, p.threads, smem, st>>>(p.d_ops, (p.nops + PG_BLOCK - 1) / PG_BLOCK, p.d_tab, a, p.tmem_cols,
                                                jtol, jtol64, max_sweeps, sweeps, err);
 }
 
-template cudaError_t pg_setup<float>();
-template cudaError_t pg_setup<double>();
-template bool pg_is_set_up<float>();
-template bool pg_is_set_up<double>();
 template void pg_launch<float>(const PgProgram&, const PgArgs&, float, double, int, unsigned long long*, int*, int,
                                cudaStream_t);
 template void pg_launch<double>(const PgProgram&, const PgArgs&, double, double, int, unsigned long long*, int*, int,

@@ -111,12 +111,6 @@ struct PgProgram {
 template <typename T>
 void pg_launch(const PgProgram& p, const PgArgs& a, T jtol, double jtol64, int max_sweeps, unsigned long long* sweeps,
                int* err, int sms, cudaStream_t st);
-template <typename T>
-cudaError_t pg_setup();
-// Whether pg_setup() has run on this device: the attributes of the kernels (forty of them) are set
-// by the first context and found by the others, for the price of one query.
-template <typename T>
-bool pg_is_set_up();
 
 constexpr size_t PG_STATIC = 5 * 1024;        // PgShared and the system's share
 constexpr size_t PG_SMEM = 227 * 1024;
