@@ -1,5 +1,5 @@
-"""Kernel attributes are set by the first context and found by the others: contexts made and freed in
-other orders, precisions and threads launch kernels of more than 48 KB of shared memory."""
+"""Shared-memory limits are set by the launches that need them: contexts of several threads, made and
+freed at the same time, launch kernels of more than 48 KB of shared memory on both routes."""
 import threading
 
 import numpy as np
